@@ -27,12 +27,12 @@ size_t align_up(size_t v) { return (v + kAlign - 1) & ~(kAlign - 1); }
 
 
 struct Layout {
-  size_t counters, cpid, fq0, fq1, eq0, eq1, dq0, dq1, nz_cell, nz_start, tile_nz, scan_bsum,
-      scan_bnz, tmp_grid, tmp_wsum, obs_density, obs_marg, obs_col, obs_scalar, rec_cell,
+  size_t counters, cpid, fq0, fq1, eq0, eq1, dq0, dq1, nz_cell, nz_start, tile_nz, scan_sub,
+      scan_grp, scan_list, tmp_grid, tmp_wsum, obs_density, obs_marg, obs_col, obs_scalar, rec_cell,
       rec_a, keep0, keep1, res0, res1, ucnt, guide, binst, dpre, bguide, seg_counts, cnt_save, tabs,
       cinst, obs_red, tab_A, tab_xmax, tab_xi0, tab_xi1, tab_cdf0, tab_cdf1, tab_guide0,
       tab_guide1, dgrid0, dgrid1, tnz_cell, tnz_start, tnz_tau, ttile_nz, total;
-  long long qcap, ecap, dcap, rec_cap, scan_blocks, tile_cap;
+  long long qcap, ecap, dcap, rec_cap, scan_blocks, scan_list_cap, tile_cap;
 };
 
 // ninst = 0: a plain run (config->n_alpha is used); ninst >= 1: a batch.
@@ -126,8 +126,10 @@ Layout layout(const wbrw_config* c, int ninst, long long capacity) {
   L.nz_cell = take((size_t)nh * 4);
   L.nz_start = take((size_t)nh * 8);
   L.tile_nz = take((size_t)L.tile_cap * 4);
-  L.scan_bsum = take((size_t)(L.scan_blocks + 1) * 8);
-  L.scan_bnz = take((size_t)(L.scan_blocks + 1) * 4);
+  L.scan_sub = take((size_t)L.scan_blocks * sizeof(ScanPair));
+  L.scan_grp = take((size_t)kScanGroups * sizeof(ScanPair));
+  L.scan_list_cap = L.tile_cap / kDenseTiles + 1;
+  L.scan_list = take((size_t)L.scan_list_cap * 4);
   L.tmp_grid = take((size_t)nh * 4);
   L.tmp_wsum = take((size_t)nh * 8);
   L.obs_density = take((size_t)c->nx * c->nk * 8);
@@ -690,8 +692,10 @@ wbrw_status create(const wbrw_config* config, const wbrw_potential* pot, int nin
   c->nz_start = (unsigned long long*)(base + L.nz_start);
   c->tile_nz = (uint32_t*)(base + L.tile_nz);
   c->tile_cap = L.tile_cap;
-  c->scan_bsum = (unsigned long long*)(base + L.scan_bsum);
-  c->scan_bnz = (unsigned int*)(base + L.scan_bnz);
+  c->scan_sub = (ScanPair*)(base + L.scan_sub);
+  c->scan_grp = (ScanPair*)(base + L.scan_grp);
+  c->scan_list = (uint32_t*)(base + L.scan_list);
+  c->scan_list_cap = (unsigned)L.scan_list_cap;
   c->scan_blocks = L.scan_blocks;
   c->tmp_grid = (int*)(base + L.tmp_grid);
   c->tmp_wsum = (long long*)(base + L.tmp_wsum);

@@ -118,170 +118,492 @@ __device__ unsigned long long block_exscan(unsigned long long v,
 // ---------------------------------------------------------------------------
 // Histogram -> regeneration plan (Alg. 3 without rounding): n_nu = |c_nu|,
 // exclusive scan over cells, compact list of the nonzero cells with their
-// first slot.  Three passes over tiles of kScanTile cells.
+// first slot, and the first nonzero cell of every 32-slot tile.  The cells
+// are cut into sub-tiles of kScanTile; k_plan_a sums each (one read of the
+// histogram), its last block to finish scans the sums of the blocks, and
+// k_plan_c writes the plan of each sub-tile that holds anything.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kBlock) k_cells_a(const int* grid, long long nh,
-                                                    unsigned long long* bsum,
-                                                    unsigned int* bnz) {
-  __shared__ unsigned long long red[kBlock / 32 + 1];
-  const long long base = (long long)blockIdx.x * kScanTile + (long long)threadIdx.x * kScanItems;
-  unsigned long long s = 0, z = 0;
-#pragma unroll
-  for (int i = 0; i < kScanItems; ++i) {
-    const long long c = base + i;
-    if (c < nh) {
-      const int v = grid[c];
-      s += (unsigned long long)(v < 0 ? -(long long)v : (long long)v);
-      z += v != 0;
-    }
+// Sum of v over the warp, modulo 2^64: three hardware reductions of 22-bit
+// pieces (each sum below 2^27).
+__device__ __forceinline__ unsigned long long warp_sum(unsigned long long v) {
+  const unsigned a = __reduce_add_sync(0xFFFFFFFFu, (unsigned)v & 0x3FFFFFu);
+  const unsigned b = __reduce_add_sync(0xFFFFFFFFu, (unsigned)(v >> 22) & 0x3FFFFFu);
+  const unsigned c = __reduce_add_sync(0xFFFFFFFFu, (unsigned)(v >> 44));
+  return (unsigned long long)a + ((unsigned long long)b << 22) + ((unsigned long long)c << 44);
+}
+
+// The instance of global cell nu (< 2^30) when every instance owns nhi
+// cells: floor(nu / nhi) from one multiply by mag = ceil(2^40 / nhi) (whose
+// estimate exceeds the quotient by at most one, since nu (mag - 2^40 / nhi)
+// < 2^-10 2^40) and one correction, instead of an integer division.
+__device__ __forceinline__ unsigned long long inst_magic(int nhi) {
+  return ((1ull << 40) + (unsigned long long)nhi - 1ull) / (unsigned long long)nhi;
+}
+__device__ __forceinline__ unsigned inst_of_cell(unsigned nu, int nhi, unsigned long long mag) {
+  unsigned q = (unsigned)(((unsigned long long)nu * mag) >> 40);
+  if (q * (unsigned)nhi > nu) --q;
+  return q;
+}
+
+// What a plan is made from: the signed histogram ...
+struct PlanGrid {
+  const int* grid;
+  uint32_t* nz_cell;
+  using V = int;
+  __device__ V load(long long c) const { return grid[c]; }
+  __device__ static V none() { return 0; }
+  __device__ static unsigned long long count(V v) {
+    return (unsigned long long)(v < 0 ? -(long long)v : (long long)v);
   }
-  unsigned long long ts, tz;
-  block_exscan(s, red, ts);
-  block_exscan(z, red, tz);
+  __device__ void put(unsigned idx, long long c, V v, unsigned long long) const {
+    nz_cell[idx] = (uint32_t)c | (v < 0 ? 0x80000000u : 0u);
+  }
+};
+
+// ... or the tangent histogram: cell nu carries n_nu = ceil(max(|D_H|, |D_w|)
+// / quantum) tangent particles with tau = D_nu / n_nu each.  A quantum of
+// 2^qs units divides by a shift (a 64-bit division costs about a hundred
+// instructions a cell); qs < 0: any other quantum.
+struct PlanTangent {
+  const long long *dH, *dw;
+  long long q;
+  int qs;
+  uint32_t* nz_cell;
+  double* nz_tau;
+  struct V {
+    long long h, w;
+    unsigned long long n;
+  };
+  __device__ V load(long long c) const {
+    V v;
+    v.h = dH[c];
+    v.w = dw[c];
+    const long long a = v.h < 0 ? -v.h : v.h, b = v.w < 0 ? -v.w : v.w;
+    const long long m = a > b ? a : b;
+    v.n = m == 0 ? 0ull
+                 : (unsigned long long)(qs >= 0 ? (m + q - 1) >> qs : (m + q - 1) / q);
+    return v;
+  }
+  __device__ static V none() { return V{0, 0, 0ull}; }
+  __device__ static unsigned long long count(const V& v) { return v.n; }
+  __device__ void put(unsigned idx, long long c, const V& v, unsigned long long n) const {
+    nz_cell[idx] = (uint32_t)c;
+    nz_tau[2 * (size_t)idx] = __ddiv_rn(__dmul_rn((double)v.h, 1.0 / 4294967296.0), (double)n);
+    nz_tau[2 * (size_t)idx + 1] = __ddiv_rn(__dmul_rn((double)v.w, 1.0 / 4294967296.0), (double)n);
+  }
+};
+
+// Whether the calling block is the last of the grid to arrive (its earlier
+// writes and every other block's are then visible to it); it leaves the
+// ticket at zero for the next launch.  No block waits.
+__device__ bool last_block(unsigned* ticket) {
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
   if (threadIdx.x == 0) {
-    bsum[blockIdx.x] = ts;
-    bnz[blockIdx.x] = (unsigned int)tz;
+    last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    if (last) *ticket = 0u;
+  }
+  __syncthreads();
+  if (last) __threadfence();
+  return last;
+}
+
+// Exclusive prefix of the block sums in place (ng <= kScanGroups entries, a
+// few per thread), by one block; the totals are returned to every thread.
+__device__ void scan_groups(ScanPair* grp, int ng, unsigned long long* red,
+                            unsigned long long& ta, unsigned long long& tb) {
+  constexpr int kPer = (kScanGroups + kBlock - 1) / kBlock;
+  ScanPair v[kPer];
+  unsigned long long a = 0, b = 0;
+#pragma unroll
+  for (int i = 0; i < kPer; ++i) {
+    const int g = threadIdx.x * kPer + i;
+    v[i].a = g < ng ? __ldcg(&grp[g].a) : 0ull;
+    v[i].b = g < ng ? __ldcg(&grp[g].b) : 0ull;
+    a += v[i].a;
+    b += v[i].b;
+  }
+  unsigned long long ea = block_exscan(a, red, ta);
+  unsigned long long eb = block_exscan(b, red, tb);
+#pragma unroll
+  for (int i = 0; i < kPer; ++i) {
+    const int g = threadIdx.x * kPer + i;
+    if (g < ng) {
+      grp[g].a = ea;
+      grp[g].b = eb;
+    }
+    ea += v[i].a;
+    eb += v[i].b;
   }
 }
 
-// which = 0: the plan of the signed particles; 1: the tangent plan.
-__global__ void __launch_bounds__(kBlock) k_cells_b(unsigned long long* bsum,
-                                                    unsigned int* bnz,
-                                                    long long nb, Counters* c,
-                                                    long long tile_cap,
-                                                    unsigned long long* inst_end, int which) {
-  __shared__ unsigned long long red[kBlock / 32 + 1];
-  unsigned long long carry_s = 0, carry_z = 0;
-  for (long long b0 = 0; b0 < nb; b0 += kBlock) {
-    const long long b = b0 + threadIdx.x;
-    const unsigned long long s = b < nb ? bsum[b] : 0, z = b < nb ? bnz[b] : 0;
-    unsigned long long ts, tz;
-    const unsigned long long es = block_exscan(s, red, ts);
-    const unsigned long long ez = block_exscan(z, red, tz);
-    if (b < nb) {
-      bsum[b] = carry_s + es;
-      bnz[b] = (unsigned int)(carry_z + ez);
+// Block b sums the sub-tiles [b per, (b + 1) per): their slots and nonzero
+// cells, and the running sums before each within the block.  which = 0: the
+// plan of the signed particles; 1: the tangent plan.
+// Memory bound: one read of the cells, eight coalesced loads a thread in
+// flight.  With the scan of the block sums done by the last block there is
+// no third launch, and no block ever scans more than kScanGroups sums (one
+// thread-block scanning 19200 tile sums took 76 us of a 256-instance batch).
+template <class S>
+__global__ void __launch_bounds__(kBlock) k_plan_a(const S src, long long nh, int nsub, int per,
+                                                   ScanSub* sub, ScanPair* grp, Counters* c,
+                                                   long long tile_cap,
+                                                   unsigned long long* inst_end, int which) {
+  constexpr int kW = kBlock / 32;
+  __shared__ unsigned long long red[kW + 1];
+  __shared__ unsigned long long ss[2][kW];
+  __shared__ unsigned sz[2][kW];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int t0 = blockIdx.x * per, t1 = min(t0 + per, nsub);
+  unsigned long long run_s = 0;
+  unsigned run_z = 0;
+  for (int t = t0; t < t1; ++t) {
+    const long long base = (long long)t * kScanTile + threadIdx.x;
+    typename S::V v[kScanItems];
+#pragma unroll
+    for (int i = 0; i < kScanItems; ++i) {
+      const long long cell = base + i * kBlock;
+      v[i] = cell < nh ? src.load(cell) : S::none();
     }
-    carry_s += ts;
-    carry_z += tz;
+    unsigned long long s = 0;
+    unsigned z = 0;
+#pragma unroll
+    for (int i = 0; i < kScanItems; ++i) {
+      const unsigned long long n = S::count(v[i]);
+      s += n;
+      z += n != 0;
+    }
+    z = __reduce_add_sync(0xFFFFFFFFu, z);
+    s = z ? warp_sum(s) : 0ull;
+    const int k = (t - t0) & 1;  // two buffers: one barrier per sub-tile
+    if (lane == 0) {
+      ss[k][wid] = s;
+      sz[k][wid] = z;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      unsigned long long bs = 0;
+      unsigned bz = 0;
+#pragma unroll
+      for (int i = 0; i < kW; ++i) {
+        bs += ss[k][i];
+        bz += sz[k][i];
+      }
+      sub[t] = ScanSub{run_s, run_z, bz};
+      run_s += bs;
+      run_z += bz;
+    }
   }
+  if (threadIdx.x == 0) grp[blockIdx.x] = ScanPair{run_s, run_z};
+  if (!last_block(&c->scan_ticket)) return;
+  unsigned long long ts, tz;
+  scan_groups(grp, gridDim.x, red, ts, tz);
   if (threadIdx.x == 0) {
     if (which) {
-      c->tan_total = carry_s;
-      c->tan_nz = carry_z;
+      c->tan_total = ts;
+      c->tan_nz = tz;
     } else {
-      c->regen_total = carry_s;
-      c->nz_count = carry_z;
+      c->regen_total = ts;
+      c->nz_count = tz;
     }
-    *inst_end = carry_s;
-    if (carry_s > (unsigned long long)tile_cap * 32ull) atomicOr(&c->err, ERR_CAP_PARTICLES);
+    *inst_end = ts;
+    c->scan_dense = 0;
+    if (ts > (unsigned long long)tile_cap * 32ull) atomicOr(&c->err, ERR_CAP_PARTICLES);
   }
 }
 
-// Also records the first slot of each instance (cells i nhi .. (i+1) nhi - 1
-// belong to instance i) in inst_slot.
-__global__ void __launch_bounds__(kBlock) k_cells_c(const int* grid, long long nh,
-                                                    const unsigned long long* bsum,
-                                                    const unsigned int* bnz,
-                                                    uint32_t* nz_cell,
-                                                    unsigned long long* nz_start,
-                                                    uint32_t* tile_nz, long long tile_cap,
-                                                    long long nhi,
-                                                    unsigned long long* inst_slot) {
-  __shared__ unsigned long long red[kBlock / 32 + 1];
-  const long long base = (long long)blockIdx.x * kScanTile + (long long)threadIdx.x * kScanItems;
-  int v[kScanItems];
-  unsigned long long s = 0, z = 0;
-#pragma unroll
-  for (int i = 0; i < kScanItems; ++i) {
-    const long long c = base + i;
-    v[i] = c < nh ? grid[c] : 0;
-    s += (unsigned long long)(v[i] < 0 ? -(long long)v[i] : (long long)v[i]);
-    z += v[i] != 0;
-  }
-  unsigned long long ts, tz;
-  unsigned long long os = block_exscan(s, red, ts) + bsum[blockIdx.x];
-  unsigned long long oz = block_exscan(z, red, tz) + bnz[blockIdx.x];
-  long long next_inst = (base + nhi - 1) / nhi * nhi;  // first instance boundary >= base
+// The plan entries of one warp's 256 cells (32 consecutive ones per item)
+// from slot S and plan position Z on, and the tiles whose first slot falls
+// into cells of fewer than kDenseTiles tiles: 32 tiles a step, each lane
+// finding its tile's cell by a search in the running sums of their runs.  The runs of equal entries of denser cells are left to k_plan_t
+// (their plan positions go to its list) or, without a list, written here.
+// W: the type of sums within a sub-tile.
+template <class W, class S>
+__device__ __forceinline__ void plan_items(const S& src, long long wbase,
+                                           long long nh, unsigned long long slot, unsigned z,
+                                           bool bounds, int nhi, unsigned long long mag,
+                                           unsigned long long* nz_start, uint32_t* tile_nz,
+                                           unsigned long long tile_cap, uint32_t* list,
+                                           unsigned* nlist, unsigned list_cap,
+                                           unsigned long long* inst_slot) {
   const int lane = threadIdx.x & 31;
-#pragma unroll
+#pragma unroll 1
   for (int i = 0; i < kScanItems; ++i) {
-    if (base + i == next_inst && next_inst < nh) {
-      inst_slot[next_inst / nhi] = os;
-      next_inst += nhi;
+    const long long cell = wbase + 32 * i + lane;
+    const typename S::V v = cell < nh ? src.load(cell) : S::none();  // from L1: just read
+    const unsigned long long n = S::count(v);
+    const unsigned bal = __ballot_sync(0xFFFFFFFFu, n != 0);
+    W inc = (W)n;
+    if (bal) {
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const W u = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+        if (lane >= o) inc += u;
+      }
     }
-    // every 32-slot tile whose first slot falls in this cell starts here:
-    // tiles [t0, t1) (tile indices fit 32 bits: tile_cap <= capacity / 32 + 2)
-    unsigned t0 = 0, t1 = 0;
-    const uint32_t val = (uint32_t)oz;
-    if (v[i] != 0) {
-      const unsigned long long m = (unsigned long long)(v[i] < 0 ? -(long long)v[i] : (long long)v[i]);
-      nz_cell[oz] = (uint32_t)(base + i) | (v[i] < 0 ? 0x80000000u : 0u);
-      nz_start[oz] = os;
-      t0 = (unsigned)min((os + 31) >> 5, (unsigned long long)tile_cap);
-      t1 = (unsigned)min((os + m + 31) >> 5, (unsigned long long)tile_cap);
-      ++oz;
-      os += m;
+    const unsigned long long start = slot + (unsigned long long)(W)(inc - (W)n);
+    if (bounds && cell < nh) {  // the first cell of an instance
+      const unsigned q = inst_of_cell((unsigned)cell, nhi, mag);
+      if ((long long)q * nhi == cell) inst_slot[q] = start;
     }
-    // the warp writes each lane's tile range in turn, 32 consecutive
-    // entries per store (a dense cell spans many tiles)
-    for (unsigned pend = __ballot_sync(0xFFFFFFFFu, t1 > t0); pend; pend &= pend - 1) {
-      const int src = __ffs(pend) - 1;
-      const unsigned a = __shfl_sync(0xFFFFFFFFu, t0, src), b = __shfl_sync(0xFFFFFFFFu, t1, src);
-      const uint32_t w = __shfl_sync(0xFFFFFFFFu, val, src);
-      for (unsigned t = a + lane; t < b; t += 32) tile_nz[t] = w;
+    if (!bal) continue;
+    if (n) {
+      const unsigned idx = z + __popc(bal & ((1u << lane) - 1u));
+      src.put(idx, cell, v, n);
+      nz_start[idx] = start;
     }
+    const unsigned long long tot = __shfl_sync(0xFFFFFFFFu, inc, 31);
+    // this lane's run of tiles [a, b); the runs of the cells that are not
+    // dense one after the other, 32 tiles a step
+    const unsigned a = (unsigned)min((start + 31) >> 5, tile_cap);
+    const unsigned b = n ? (unsigned)min((start + n + 31) >> 5, tile_cap) : a;
+    const unsigned dense = __ballot_sync(0xFFFFFFFFu, b - a >= (unsigned)kDenseTiles);
+    const unsigned len = (dense >> lane) & 1u ? 0u : b - a;
+    unsigned run = len;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned u = __shfl_up_sync(0xFFFFFFFFu, run, o);
+      if (lane >= o) run += u;
+    }
+    const unsigned light = __shfl_sync(0xFFFFFFFFu, run, 31);
+    const unsigned off = a - (run - len);
+    for (unsigned kb = 0; kb < light; kb += 32) {
+      const unsigned k = kb + lane;
+      int o = 0;  // the cells whose runs end at or before entry k
+#pragma unroll
+      for (int st = 16; st > 0; st >>= 1) {
+        const unsigned u = __shfl_sync(0xFFFFFFFFu, run, o + st - 1);
+        if (u <= k) o += st;
+      }
+      const unsigned t = __shfl_sync(0xFFFFFFFFu, off, o) + k;
+      if (k < light) tile_nz[t] = z + __popc(bal & ((1u << o) - 1u));
+    }
+    if (dense) {
+      if (list) {
+        unsigned at = 0;
+        if (lane == 0) at = atomicAdd(nlist, (unsigned)__popc(dense));
+        at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(dense & ((1u << lane) - 1u));
+        if (((dense >> lane) & 1u) && at < list_cap)
+          list[at] = z + __popc(bal & ((1u << lane) - 1u));
+      } else {
+        for (unsigned pend = dense; pend; pend &= pend - 1) {
+          const int o = __ffs(pend) - 1;
+          const unsigned ta = __shfl_sync(0xFFFFFFFFu, a, o), te = __shfl_sync(0xFFFFFFFFu, b, o);
+          for (unsigned t = ta + lane; t < te; t += 32)
+            tile_nz[t] = z + __popc(bal & ((1u << o) - 1u));
+        }
+      }
+    }
+    slot += tot;
+    z += __popc(bal);
+  }
+}
+
+// Writes the plan.  Also records the first slot of each instance (cells
+// i nhi .. (i+1) nhi - 1 belong to instance i) in inst_slot.  Sub-tiles
+// without a particle are skipped (k_plan_a counted their nonzero cells): the
+// histograms are sparse, so most of the second read falls away.  A warp
+// takes 256 cells as eight coalesced loads of 32.
+template <class S>
+__global__ void __launch_bounds__(kBlock) k_plan_c(const S src, long long nh, int nsub, int per,
+                                                   const ScanSub* sub, const ScanPair* grp,
+                                                   unsigned long long* nz_start,
+                                                   uint32_t* tile_nz, long long tile_cap,
+                                                   uint32_t* list, unsigned* nlist,
+                                                   unsigned list_cap, int nhi, int ninst,
+                                                   unsigned long long* inst_slot) {
+  constexpr int kW = kBlock / 32;
+  __shared__ unsigned long long ss[2][kW];
+  __shared__ unsigned sz[2][kW];
+  const unsigned long long mag = inst_magic(nhi);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  int k = 0;
+  for (int t = blockIdx.x; t < nsub; t += gridDim.x) {
+    const ScanSub st = sub[t];
+    const ScanPair g = grp[t / per];
+    const unsigned long long base_s = g.a + st.s;
+    const long long base = (long long)t * kScanTile;
+    const long long end = min(base + kScanTile, nh);
+    if (st.nz == 0) {
+      for (long long i = (base + nhi - 1) / nhi + threadIdx.x; i < ninst && i * nhi < end;
+           i += kBlock)
+        inst_slot[i] = base_s;
+      continue;
+    }
+    const long long wbase = base + wid * (kScanTile / kW);
+    unsigned long long s = 0;
+    unsigned z = 0;
+#pragma unroll
+    for (int i = 0; i < kScanItems; ++i) {
+      const long long cell = wbase + 32 * i + lane;
+      const unsigned long long n = S::count(cell < nh ? src.load(cell) : S::none());
+      s += n;
+      z += n != 0;
+    }
+    s = warp_sum(s);
+    z = __reduce_add_sync(0xFFFFFFFFu, z);
+    if (lane == 0) {
+      ss[k][wid] = s;
+      sz[k][wid] = z;
+    }
+    __syncthreads();
+    unsigned long long pre_s = 0, all_s = 0;
+    unsigned pre_z = 0;
+#pragma unroll
+    for (int i = 0; i < kW; ++i) {
+      if (i < wid) {
+        pre_s += ss[k][i];
+        pre_z += sz[k][i];
+      }
+      all_s += ss[k][i];
+    }
+    k ^= 1;  // two buffers: one barrier per sub-tile
+    const bool bounds = ninst > 1 || t == 0;
+    const unsigned z0 = (unsigned)g.b + st.z + pre_z;
+    if (z == 0 && !bounds) continue;
+    if (all_s < (1ull << 32))
+      plan_items<unsigned>(src, wbase, nh, base_s + pre_s, z0, bounds, nhi, mag, nz_start,
+                           tile_nz, (unsigned long long)tile_cap, list, nlist, list_cap,
+                           inst_slot);
+    else
+      plan_items<unsigned long long>(src, wbase, nh, base_s + pre_s, z0, bounds, nhi, mag,
+                                     nz_start, tile_nz, (unsigned long long)tile_cap, list, nlist,
+                                     list_cap, inst_slot);
+  }
+}
+
+// The tiles of the dense cells: a warp each, so that the few columns that hold most of a packet's slots are spread over
+// the whole chip.  (Written by the warps that scan those columns, the table
+// of 1.4e8 particles on 1200 x 512 cells took 49 us.)
+__global__ void __launch_bounds__(kBlock) k_plan_t(const Counters* c, int which,
+                                                   const unsigned long long* nz_start,
+                                                   const uint32_t* list, unsigned list_cap,
+                                                   uint32_t* tile_nz, long long tile_cap) {
+  const int lane = threadIdx.x & 31;
+  const unsigned long long total = which ? c->tan_total : c->regen_total;
+  const unsigned nz = (unsigned)(which ? c->tan_nz : c->nz_count);
+  const unsigned n = min(c->scan_dense, list_cap);
+  const unsigned w = (blockIdx.x * kBlock + threadIdx.x) >> 5, nw = (gridDim.x * kBlock) >> 5;
+  if (n == 0) return;
+  const unsigned parts = max(1u, nw / n);  // warps per cell when there are few
+  for (unsigned j = w; j < n * parts; j += nw) {
+    const uint32_t idx = list[j % n];
+    const unsigned long long s0 = nz_start[idx], s1 = idx + 1 < nz ? nz_start[idx + 1] : total;
+    const unsigned a = (unsigned)min((s0 + 31) >> 5, (unsigned long long)tile_cap);
+    const unsigned b = (unsigned)min((s1 + 31) >> 5, (unsigned long long)tile_cap);
+    for (unsigned t = a + 32u * (j / n) + lane; t < b; t += 32u * parts) tile_nz[t] = idx;
   }
 }
 
 // ---------------------------------------------------------------------------
-// In-place inclusive scan of a u64 array (per-cell bootstrap residuals).
+// In-place inclusive scans of the per-cell bootstrap residuals of both sides:
+// k_pre_a sums each sub-tile and scans the block sums as k_plan_a, k_pre_c
+// writes the prefixes.  (One launch pair for both sides; three launches per
+// side before.)
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kBlock) k_u64_a(const unsigned long long* a, long long n,
-                                                  unsigned long long* bsum) {
-  __shared__ unsigned long long red[kBlock / 32 + 1];
-  const long long base = (long long)blockIdx.x * kScanTile + (long long)threadIdx.x * kScanItems;
-  unsigned long long s = 0;
+__global__ void __launch_bounds__(kBlock) k_pre_a(const unsigned long long* a,
+                                                  const unsigned long long* b, long long n,
+                                                  int nsub, int per, ScanPair* sub, ScanPair* grp,
+                                                  Counters* c) {
+  constexpr int kW = kBlock / 32;
+  __shared__ unsigned long long red[kW + 1];
+  __shared__ unsigned long long sa[2][kW], sb[2][kW];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int t0 = blockIdx.x * per, t1 = min(t0 + per, nsub);
+  unsigned long long run_a = 0, run_b = 0;
+  for (int t = t0; t < t1; ++t) {
+    const long long base = (long long)t * kScanTile + threadIdx.x;
+    unsigned long long va = 0, vb = 0;
 #pragma unroll
-  for (int i = 0; i < kScanItems; ++i)
-    if (base + i < n) s += a[base + i];
-  unsigned long long t;
-  block_exscan(s, red, t);
-  if (threadIdx.x == 0) bsum[blockIdx.x] = t;
+    for (int i = 0; i < kScanItems; ++i) {
+      const long long cell = base + i * kBlock;
+      if (cell < n) {
+        va += a[cell];
+        vb += b[cell];
+      }
+    }
+    va = warp_sum(va);
+    vb = warp_sum(vb);
+    const int k = (t - t0) & 1;
+    if (lane == 0) {
+      sa[k][wid] = va;
+      sb[k][wid] = vb;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      sub[t] = ScanPair{run_a, run_b};
+#pragma unroll
+      for (int i = 0; i < kW; ++i) {
+        run_a += sa[k][i];
+        run_b += sb[k][i];
+      }
+    }
+  }
+  if (threadIdx.x == 0) grp[blockIdx.x] = ScanPair{run_a, run_b};
+  if (!last_block(&c->scan_ticket)) return;
+  unsigned long long ta, tb;
+  scan_groups(grp, gridDim.x, red, ta, tb);
+  if (threadIdx.x == 0) {
+    c->boot_R[0] = ta;
+    c->boot_R[1] = tb;
+  }
 }
 
-__global__ void __launch_bounds__(kBlock) k_u64_b(unsigned long long* bsum, long long nb,
-                                                  unsigned long long* total) {
-  __shared__ unsigned long long red[kBlock / 32 + 1];
-  unsigned long long carry = 0;
-  for (long long b0 = 0; b0 < nb; b0 += kBlock) {
-    const long long b = b0 + threadIdx.x;
-    const unsigned long long s = b < nb ? bsum[b] : 0;
-    unsigned long long t;
-    const unsigned long long e = block_exscan(s, red, t);
-    if (b < nb) bsum[b] = carry + e;
-    carry += t;
-  }
-  if (threadIdx.x == 0) *total = carry;
-}
-
-__global__ void __launch_bounds__(kBlock) k_u64_c(unsigned long long* a, long long n,
-                                                  const unsigned long long* bsum) {
-  __shared__ unsigned long long red[kBlock / 32 + 1];
-  const long long base = (long long)blockIdx.x * kScanTile + (long long)threadIdx.x * kScanItems;
-  unsigned long long v[kScanItems];
-  unsigned long long s = 0;
+__global__ void __launch_bounds__(kBlock) k_pre_c(unsigned long long* a, unsigned long long* b,
+                                                  long long n, int nsub, int per,
+                                                  const ScanPair* sub, const ScanPair* grp) {
+  constexpr int kW = kBlock / 32;
+  __shared__ unsigned long long sa[2][kW], sb[2][kW];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  int k = 0;
+  for (int t = blockIdx.x; t < nsub; t += gridDim.x) {
+    const ScanPair st = sub[t], g = grp[t / per];
+    const long long wbase = (long long)t * kScanTile + wid * (kScanTile / kW);
+    unsigned long long va[kScanItems], vb[kScanItems], ta = 0, tb = 0;
 #pragma unroll
-  for (int i = 0; i < kScanItems; ++i) {
-    v[i] = base + i < n ? a[base + i] : 0;
-    s += v[i];
-  }
-  unsigned long long t;
-  unsigned long long run = block_exscan(s, red, t) + bsum[blockIdx.x];
+    for (int i = 0; i < kScanItems; ++i) {
+      const long long cell = wbase + 32 * i + lane;
+      va[i] = cell < n ? a[cell] : 0ull;
+      vb[i] = cell < n ? b[cell] : 0ull;
+      ta += va[i];
+      tb += vb[i];
+    }
+    ta = warp_sum(ta);
+    tb = warp_sum(tb);
+    if (lane == 0) {
+      sa[k][wid] = ta;
+      sb[k][wid] = tb;
+    }
+    __syncthreads();
+    unsigned long long ra = g.a + st.a, rb = g.b + st.b;
+    for (int i = 0; i < wid; ++i) {
+      ra += sa[k][i];
+      rb += sb[k][i];
+    }
+    k ^= 1;
 #pragma unroll
-  for (int i = 0; i < kScanItems; ++i) {
-    run += v[i];
-    if (base + i < n) a[base + i] = run;
+    for (int i = 0; i < kScanItems; ++i) {
+      const long long cell = wbase + 32 * i + lane;
+      unsigned long long ia = va[i], ib = vb[i];
+      if (__any_sync(0xFFFFFFFFu, (ia | ib) != 0ull)) {
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const unsigned long long ua = __shfl_up_sync(0xFFFFFFFFu, ia, o);
+          const unsigned long long ub = __shfl_up_sync(0xFFFFFFFFu, ib, o);
+          if (lane >= o) {
+            ia += ua;
+            ib += ub;
+          }
+        }
+      }
+      if (cell < n) {
+        a[cell] = ra + ia;
+        b[cell] = rb + ib;
+      }
+      ra += __shfl_sync(0xFFFFFFFFu, ia, 31);
+      rb += __shfl_sync(0xFFFFFFFFu, ib, 31);
+    }
   }
 }
 
@@ -385,19 +707,6 @@ __global__ void __launch_bounds__(kBlock) k_boot_unit(Counters* c, const int* uc
     block_exscan(s ? ks1 : ks0, red, t);
     if (threadIdx.x == 0 && t) atomicAdd(&c->boot_keep[s], t);
   }
-}
-
-// The instance of global cell nu (< 2^30) when every instance owns nhi
-// cells: floor(nu / nhi) from one multiply by mag = ceil(2^40 / nhi) (whose
-// estimate exceeds the quotient by at most one, since nu (mag - 2^40 / nhi)
-// < 2^-10 2^40) and one correction, instead of an integer division.
-__device__ __forceinline__ unsigned long long inst_magic(int nhi) {
-  return ((1ull << 40) + (unsigned long long)nhi - 1ull) / (unsigned long long)nhi;
-}
-__device__ __forceinline__ unsigned inst_of_cell(unsigned nu, int nhi, unsigned long long mag) {
-  unsigned q = (unsigned)(((unsigned long long)nu * mag) >> 40);
-  if (q * (unsigned)nhi > nu) --q;
-  return q;
 }
 
 // The offspring records' shares added to the cell tallies.  BATCH: the
@@ -1109,83 +1418,6 @@ __global__ void __launch_bounds__(kBlock) k_reduce4(const int* counts, int nx, i
   }
 }
 
-// ---------------------------------------------------------------------------
-// Tangent plan (tangent mode): cell nu carries n_nu = ceil(max(|D_H|, |D_w|)
-// / quantum) tangent particles with tau = D_nu / n_nu each.  The same three
-// passes as the plan of the signed particles.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ unsigned long long tan_count(const long long* dH, const long long* dw,
-                                                       long long c, long long q) {
-  const long long a = dH[c] < 0 ? -dH[c] : dH[c], b = dw[c] < 0 ? -dw[c] : dw[c];
-  const long long m = a > b ? a : b;
-  return m ? (unsigned long long)((m + q - 1) / q) : 0ull;
-}
-
-__global__ void __launch_bounds__(kBlock) k_tcells_a(const long long* dH, const long long* dw,
-                                                     long long nh, long long q,
-                                                     unsigned long long* bsum, unsigned int* bnz) {
-  __shared__ unsigned long long red[kBlock / 32 + 1];
-  const long long base = (long long)blockIdx.x * kScanTile + (long long)threadIdx.x * kScanItems;
-  unsigned long long s = 0, z = 0;
-  for (int i = 0; i < kScanItems; ++i) {
-    const long long c = base + i;
-    if (c < nh) {
-      const unsigned long long n = tan_count(dH, dw, c, q);
-      s += n;
-      z += n != 0;
-    }
-  }
-  unsigned long long ts, tz;
-  block_exscan(s, red, ts);
-  block_exscan(z, red, tz);
-  if (threadIdx.x == 0) {
-    bsum[blockIdx.x] = ts;
-    bnz[blockIdx.x] = (unsigned int)tz;
-  }
-}
-
-__global__ void __launch_bounds__(kBlock) k_tcells_c(const long long* dH, const long long* dw,
-                                                     long long nh, long long q,
-                                                     const unsigned long long* bsum,
-                                                     const unsigned int* bnz, uint32_t* nz_cell,
-                                                     unsigned long long* nz_start, double* nz_tau,
-                                                     uint32_t* tile_nz, long long tile_cap,
-                                                     long long nhi, unsigned long long* inst_slot) {
-  __shared__ unsigned long long red[kBlock / 32 + 1];
-  const long long base = (long long)blockIdx.x * kScanTile + (long long)threadIdx.x * kScanItems;
-  unsigned long long n[kScanItems];  // unrolled loops keep it in registers
-  unsigned long long s = 0, z = 0;
-#pragma unroll
-  for (int i = 0; i < kScanItems; ++i) {
-    const long long c = base + i;
-    n[i] = c < nh ? tan_count(dH, dw, c, q) : 0ull;
-    s += n[i];
-    z += n[i] != 0;
-  }
-  unsigned long long ts, tz;
-  unsigned long long os = block_exscan(s, red, ts) + bsum[blockIdx.x];
-  unsigned long long oz = block_exscan(z, red, tz) + bnz[blockIdx.x];
-  long long next_inst = (base + nhi - 1) / nhi * nhi;
-#pragma unroll
-  for (int i = 0; i < kScanItems; ++i) {
-    const long long c = base + i;
-    if (c == next_inst && next_inst < nh) {
-      inst_slot[next_inst / nhi] = os;
-      next_inst += nhi;
-    }
-    if (n[i]) {
-      nz_cell[oz] = (uint32_t)c;
-      nz_start[oz] = os;
-      nz_tau[2 * oz] = __ddiv_rn(__dmul_rn((double)dH[c], 1.0 / 4294967296.0), (double)n[i]);
-      nz_tau[2 * oz + 1] = __ddiv_rn(__dmul_rn((double)dw[c], 1.0 / 4294967296.0), (double)n[i]);
-      const unsigned long long t_end = min((os + n[i] + 31) >> 5, (unsigned long long)tile_cap);
-      for (unsigned long long t = (os + 31) >> 5; t < t_end; ++t) tile_nz[t] = (uint32_t)oz;
-      ++oz;
-      os += n[i];
-    }
-  }
-}
-
 // (dT/dH, dT/dw) of each instance (one block each): the tangent histogram
 // summed over the cells with centre x > 0, times 2^-32, over N_alpha.
 __global__ void __launch_bounds__(kBlock) k_obs_tgrad(const long long* dH, const long long* dw,
@@ -1230,22 +1462,66 @@ cudaError_t launch_zero(Ctx* c, void* p, size_t bytes) {
   return cudaMemsetAsync(p, 0, bytes, c->stream);
 }
 
-cudaError_t launch_scan_cells(Ctx* c, const int* grid) {
-  const long long nb = c->scan_blocks;
-  k_cells_a<<<(unsigned)nb, kBlock, 0, c->stream>>>(grid, c->nh, c->scan_bsum, c->scan_bnz);
-  k_cells_b<<<1, kBlock, 0, c->stream>>>(c->scan_bsum, c->scan_bnz, nb, c->cnt, c->tile_cap,
-                                         c->inst_slot + c->ninst, 0);
-  k_cells_c<<<(unsigned)nb, kBlock, 0, c->stream>>>(grid, c->nh, c->scan_bsum, c->scan_bnz,
-                                                   c->nz_cell, c->nz_start, c->tile_nz,
-                                                   c->tile_cap, c->nhi, c->inst_slot);
-  c->launches += 3;
+namespace {
+
+constexpr long long kTileInline = 1 << 16;  // tiles: 2^21 slots
+
+// The launch shape of the scans: blocks of k_*_a, sub-tiles per block.
+struct ScanShape {
+  int nsub, per, groups;
+  explicit ScanShape(const Ctx* c) {
+    nsub = (int)c->scan_blocks;  // nh < 2^30 cells: below 2^19
+    per = (nsub + kScanGroups - 1) / kScanGroups;
+    groups = (nsub + per - 1) / per;
+  }
+  int grid_c(Ctx* c) const { return min(nsub, grid_cap(c, 32)); }
+  static int min(int a, int b) { return a < b ? a : b; }
+};
+
+template <class S>
+cudaError_t launch_plan(Ctx* c, const S& src, unsigned long long* nz_start, uint32_t* tile_nz,
+                        unsigned long long* inst_slot, int which) {
+  const ScanShape sh(c);
+  // the dense cells' tiles in a launch of their own, but for contexts of few
+  // slots, whose table k_plan_c writes in less than a launch takes
+  const bool apart = c->tile_cap > kTileInline;
+  k_plan_a<S><<<sh.groups, kBlock, 0, c->stream>>>(src, c->nh, sh.nsub, sh.per,
+                                                   (ScanSub*)c->scan_sub, c->scan_grp, c->cnt,
+                                                   c->tile_cap, inst_slot + c->ninst, which);
+  k_plan_c<S><<<sh.grid_c(c), kBlock, 0, c->stream>>>(
+      src, c->nh, sh.nsub, sh.per, (const ScanSub*)c->scan_sub, c->scan_grp, nz_start, tile_nz,
+      c->tile_cap, apart ? c->scan_list : nullptr, &c->cnt->scan_dense, c->scan_list_cap,
+      (int)c->nhi, c->ninst, inst_slot);
+  c->launches += 2;
+  if (apart) {
+    k_plan_t<<<grid_cap(c, 8), kBlock, 0, c->stream>>>(c->cnt, which, nz_start, c->scan_list,
+                                                       c->scan_list_cap, tile_nz, c->tile_cap);
+    c->launches++;
+  }
   return cudaGetLastError();
+}
+
+// Inclusive prefixes of both sides' residuals, in place; the totals into
+// the counters.
+void launch_residual_prefix(Ctx* c) {
+  const ScanShape sh(c);
+  k_pre_a<<<sh.groups, kBlock, 0, c->stream>>>(c->boot_res[0], c->boot_res[1], c->nh, sh.nsub,
+                                               sh.per, c->scan_sub, c->scan_grp, c->cnt);
+  k_pre_c<<<sh.grid_c(c), kBlock, 0, c->stream>>>(c->boot_res[0], c->boot_res[1], c->nh, sh.nsub,
+                                                  sh.per, c->scan_sub, c->scan_grp);
+  c->launches += 2;
+}
+
+}  // namespace
+
+cudaError_t launch_scan_cells(Ctx* c, const int* grid) {
+  return launch_plan(c, PlanGrid{grid, c->nz_cell}, c->nz_start, c->tile_nz, c->inst_slot, 0);
 }
 
 // sp2 in a batch: every instance bootstrapped on its own (Alg. 2 per
 // instance and side), in the same launches.
 static cudaError_t launch_boot_batch(Ctx* c, int epoch_delta) {
-  const long long nh = c->nh, nb = c->scan_blocks;
+  const long long nh = c->nh;
   const int ni = c->ninst, nhi = (int)c->nhi;
   const uint32_t key0 = (uint32_t)c->cfg.seed, key1 = (uint32_t)(c->cfg.seed >> 32);
   const int fx = c->cfg.precision == WBRW_FP32;
@@ -1263,12 +1539,7 @@ static cudaError_t launch_boot_batch(Ctx* c, int epoch_delta) {
   k_bootb_keep<<<grid_cap(c, 4), kBlock, 0, c->stream>>>(c->boot_inst, c->boot_keep[0],
                                                          c->boot_keep[1], nh, nhi);
   c->launches += 5;
-  for (int s = 0; s < 2; ++s) {
-    k_u64_a<<<(unsigned)nb, kBlock, 0, c->stream>>>(c->boot_res[s], nh, c->scan_bsum);
-    k_u64_b<<<1, kBlock, 0, c->stream>>>(c->scan_bsum, nb, &c->cnt->boot_R[s]);
-    k_u64_c<<<(unsigned)nb, kBlock, 0, c->stream>>>(c->boot_res[s], nh, c->scan_bsum);
-    c->launches += 3;
-  }
+  launch_residual_prefix(c);
   k_bootb_plan<<<1, kBlock, 0, c->stream>>>(c->cnt, c->boot_inst, c->boot_res[0], c->boot_res[1],
                                             ni, nhi, c->boot_dpre);
   c->launches++;
@@ -1291,7 +1562,7 @@ static cudaError_t launch_boot_batch(Ctx* c, int epoch_delta) {
 // epoch_delta), so that a captured period replays with the right streams.
 cudaError_t launch_boot(Ctx* c, int epoch_delta) {
   if (c->ninst > 1) return launch_boot_batch(c, epoch_delta);
-  const long long nh = c->nh, nb = c->scan_blocks;
+  const long long nh = c->nh;
   const uint32_t key0 = (uint32_t)c->cfg.seed, key1 = (uint32_t)(c->cfg.seed >> 32);
   const int g = grid_cap(c, 8);
   const int fx = c->cfg.precision == WBRW_FP32;
@@ -1303,12 +1574,7 @@ cudaError_t launch_boot(Ctx* c, int epoch_delta) {
       c->cnt, c->rec_cell, c->rec_a, c->rcnt, c->nseg, c->rseg, c->boot_keep[0], c->boot_keep[1],
       c->boot_res[0], c->boot_res[1], fx, nullptr, 1, (int)c->nhi);
   c->launches++;
-  for (int s = 0; s < 2; ++s) {
-    k_u64_a<<<(unsigned)nb, kBlock, 0, c->stream>>>(c->boot_res[s], nh, c->scan_bsum);
-    k_u64_b<<<1, kBlock, 0, c->stream>>>(c->scan_bsum, nb, &c->cnt->boot_R[s]);
-    k_u64_c<<<(unsigned)nb, kBlock, 0, c->stream>>>(c->boot_res[s], nh, c->scan_bsum);
-    c->launches += 3;
-  }
+  launch_residual_prefix(c);
   k_boot_guide<<<(2 * (kGuide + 1) + kBlock - 1) / kBlock, kBlock, 0, c->stream>>>(
       c->cnt, nh, c->boot_res[0], c->boot_res[1], c->boot_guide);
   k_boot_draw<<<g, kBlock, 0, c->stream>>>(
@@ -1358,17 +1624,11 @@ cudaError_t launch_transmissions(Ctx* c, const int* counts, double* out) {
 }
 
 cudaError_t launch_scan_tangent(Ctx* c) {
-  const long long nb = c->scan_blocks;
-  k_tcells_a<<<(unsigned)nb, kBlock, 0, c->stream>>>(c->dgrid[0], c->dgrid[1], c->nh, c->tquantum,
-                                                    c->scan_bsum, c->scan_bnz);
-  k_cells_b<<<1, kBlock, 0, c->stream>>>(c->scan_bsum, c->scan_bnz, nb, c->cnt, c->tile_cap,
-                                         c->tinst_slot + c->ninst, 1);
-  k_tcells_c<<<(unsigned)nb, kBlock, 0, c->stream>>>(c->dgrid[0], c->dgrid[1], c->nh, c->tquantum,
-                                                    c->scan_bsum, c->scan_bnz, c->tnz_cell,
-                                                    c->tnz_start, c->tnz_tau, c->ttile_nz,
-                                                    c->tile_cap, c->nhi, c->tinst_slot);
-  c->launches += 3;
-  return cudaGetLastError();
+  int qs = -1;
+  for (int i = 0; i < 62; ++i)
+    if (c->tquantum == (1ll << i)) qs = i;
+  const PlanTangent src{c->dgrid[0], c->dgrid[1], c->tquantum, qs, c->tnz_cell, c->tnz_tau};
+  return launch_plan(c, src, c->tnz_start, c->ttile_nz, c->tinst_slot, 1);
 }
 
 cudaError_t launch_transmission_gradients(Ctx* c) {

@@ -13,6 +13,8 @@ constexpr int kBlock = 256;      // threads per block of every particle kernel
 constexpr int kMaxChunk = 32;    // steps fused in one flight (bits of a mask)
 constexpr int kScanItems = 8;    // cells per thread in the cell scans
 constexpr int kScanTile = kBlock * kScanItems;
+constexpr int kDenseTiles = 8;   // a cell of this many 32-slot tiles is dense (k_plan_t)
+constexpr int kScanGroups = 1216;  // most blocks of a scan's first pass (eight per SM)
 constexpr int kTabGuideBits = 8;  // 4D kick rows (FP32): guide table of 2^8 buckets per row
 constexpr int kTabGuide = 1 << kTabGuideBits;
 constexpr int kGuideBits = 16;  // sp2 draws: guide table of 2^16 buckets per side
@@ -86,8 +88,20 @@ struct Counters {
   unsigned long long tan_nz;          // cells carrying tangent weight
   int per_l0;                         // the chunk's first interval
   int err;
-  int pad[2];
+  unsigned scan_ticket;               // blocks of the scan in progress that have finished
+  unsigned scan_dense;                // dense cells of the plan in progress (k_plan_t's list)
 };
+
+// Scan scratch: a sub-tile's sums before it within its block, and its
+// nonzero cells; a block's pair of sums (16 bytes each).
+struct ScanSub {
+  unsigned long long s;
+  unsigned z, nz;
+};
+struct ScanPair {
+  unsigned long long a, b;
+};
+static_assert(sizeof(ScanSub) == sizeof(ScanPair), "one scratch array serves both");
 
 // The signed bootstrap of a batch (sp2, Alg. 2 per instance and side): one
 // record per instance in device memory.  The counts and weight sums come
@@ -215,9 +229,11 @@ struct Ctx {
   unsigned long long* nz_start;
   uint32_t* tile_nz;  // first nonzero cell of each 32-slot tile of the plan
   long long tile_cap;
-  unsigned long long* scan_bsum;
-  unsigned int* scan_bnz;
-  long long scan_blocks;
+  ScanPair* scan_sub;    // per sub-tile of kScanTile cells (ScanSub in the plan's scan)
+  ScanPair* scan_grp;    // per block of the first pass
+  long long scan_blocks; // sub-tiles
+  uint32_t* scan_list;   // plan positions of the dense cells
+  unsigned scan_list_cap;
   int* tmp_grid;
   long long* tmp_wsum;
   double* obs_density;
