@@ -349,19 +349,22 @@ wbrw_status wbrw_profile_read_events(wbrw_ctx* ctx, double* total_ms,
  * switches profiling on or off captures its period again. */
 wbrw_status wbrw_graph(wbrw_ctx* ctx, int enable);
 
-/* Schedule of the periods that regenerate from the histogram under sp1 or
- * wp (sp2 periods always run launch per round), in contexts whose kernels
- * can run a period as one launch: the 2D FP32 contexts with the static
- * potential and no event log (tangent mode included) and the FP32 4D
- * contexts.  enable = 1 (the default): the first
- * wave (or waves) and every event round of a period run in one kernel
- * launch, each warp on its own candidate segments (Alg. 1 over the period,
- * the resampling of Sec. 4.3 after it).  enable = 0: the launch-per-round
+/* Schedule of the flights (a period of wbrw_run, or the intervals of
+ * wbrw_step) in contexts whose kernels can run one in one launch, every
+ * destination but sp2's records: the 2D FP32 contexts without an event log
+ * (static potential, tangent mode included, or components), the 2D FP64
+ * contexts without one (static potential, no tangents) and the FP32 4D
+ * contexts; the ones with components and the FP64 ones only if a particle's
+ * P(candidate) per interval is at most 1/2.  enable = 1 (the default): the
+ * first wave (or waves) and every event of a flight run in one kernel
+ * launch, each warp on its own candidates (Alg. 1 over the flight; the
+ * resampling of Sec. 4.3 follows).  enable = 0: the launch-per-round
  * schedule, a first-wave launch and one event launch per round.  The
  * results are the same bit for bit (random numbers are keyed by particle
- * and interval); only the launches and the time differ.  Other contexts
+ * and interval); only the launches and the time differ, and the order of
+ * offspring appended to the arrays, which is never fixed.  Other contexts
  * accept the call and always run launch per round.  Takes effect from the
- * next period; releases captured graphs (synchronises the stream).
+ * next flight; releases captured graphs (synchronises the stream).
  * WBRW_ERR_ARG for a NULL context, WBRW_ERR_STATE after a failure. */
 wbrw_status wbrw_one_launch_periods(wbrw_ctx* ctx, int enable);
 
@@ -384,10 +387,9 @@ wbrw_status wbrw_one_launch_periods(wbrw_ctx* ctx, int enable);
  *                   (those with four blocks per SM above, and the same in
  *                   tangent mode) and the FP32 4D contexts finish every such
  *                   segment in lockstep passes inside the event kernel
- *                   itself, so there event_passes changes nothing; their
- *                   regenerating sp1 and wp periods run in one launch (first
- *                   waves and event rounds together), at most three blocks
- *                   per SM.
+ *                   itself, so there event_passes changes nothing; flights
+ *                   that run in one launch (wbrw_one_launch_periods) take at
+ *                   most three blocks per SM and no passes.
  * wbrw_set_tuning takes effect from the next call and releases captured
  * graphs; out-of-range values (including blocks_per_sm above the context's
  * maximum) give WBRW_ERR_ARG. */

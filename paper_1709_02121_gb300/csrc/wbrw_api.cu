@@ -103,7 +103,9 @@ Layout layout(const wbrw_config* c, int ninst, long long capacity) {
   // per round buffer: FP32 flights queue at most one candidate interval per
   // particle, FP64 flights all of them (about one per particle per flight)
   L.ecap = c->precision == WBRW_FP32 ? L.qcap : 2 * L.qcap;
-  L.dcap = L.ecap / 4;  // deferred segments: a few per cent of the events
+  // deferred segments: a few per cent of the events; at least two passes of
+  // a one-launch period's warp
+  L.dcap = L.ecap / 4 > floor_entries ? L.ecap / 4 : floor_entries;
   L.tile_cap = capacity / 32 + 2;
   L.rec_cap = c->strategy == WBRW_SP2_BOOTSTRAP ? 4 * L.qcap : 0;
   L.scan_blocks = (nh + kScanTile - 1) / kScanTile;
@@ -685,6 +687,8 @@ wbrw_status create(const wbrw_config* config, const wbrw_potential* pot, int nin
   c->rec_cap = L.rec_cap;
   c->passes = 3;
   c->one_launch = 1;
+  c->has_log = c->buf.event_log != nullptr;
+  c->p_max = p_max;
   c->lean = c->cfg.precision == WBRW_FP32 && c->cfg.dim == 2 && ncomp == 0 && !c->buf.event_log;
   c->max_bps = drv(c)->max_bps;
   set_shape(c, c->max_bps);

@@ -62,11 +62,21 @@ __device__ __forceinline__ uint4 philox_ks(const KeySched& ks, uint32_t c0, uint
   return make_uint4(c0, c1, c2, c3);
 }
 
-__device__ __forceinline__ double u53(uint32_t a, uint32_t b) {
-  return __dmul_rn(__dadd_rn(__dmul_rn((double)(a >> 5), 67108864.0),
-                             (double)(b >> 6)),
-                   1.0 / 9007199254740992.0);
+// U53 = ((a >> 5) 2^26 + (b >> 6)) 2^-53: the 53-bit integer n, and n 2^-53,
+// which is a double exactly.  Its bits are put together by integer
+// instructions (the position of the leading one gives the exponent): FP64
+// conversions and multiplies run at 1/64 of the integer rate on this GPU,
+// and every draw of the FP64 path needs one of these.
+__device__ __forceinline__ unsigned long long n53(uint32_t a, uint32_t b) {
+  return ((unsigned long long)(a >> 5) << 26) | (b >> 6);
 }
+__device__ __forceinline__ double u53_of(unsigned long long n) {
+  const int lz = __clzll((long long)n);
+  const unsigned long long bits =
+      ((unsigned long long)(1033 - lz) << 52) | ((n << (lz - 11)) & 0xFFFFFFFFFFFFFull);
+  return n ? __longlong_as_double((long long)bits) : 0.0;
+}
+__device__ __forceinline__ double u53(uint32_t a, uint32_t b) { return u53_of(n53(a, b)); }
 __device__ __forceinline__ float u24(uint32_t a) {
   return (float)(a >> 8) * (1.0f / 16777216.0f);
 }
@@ -139,17 +149,18 @@ struct F32 {
 // TGm: the tangent mode of the 2D model: every particle also carries its
 // likelihood-ratio tangent weight (d/dH, d/dw), see do_event.
 //
-// LEANm: a run with the static potential and no event log: 1 for one
-// instance, 2 for a batch.  The kernels then leave out the time-dependent
-// components and the log writes, and for one instance the batch decode, and
-// their registers (the results are those of the general kernels, which serve
-// every other run).
+// LEANm: a run without an event log: with the static potential 1 for one
+// instance and 2 for a batch, 3 with a time-dependent one (one instance).
+// The kernels then leave out the log writes, the time-dependent components
+// (1, 2) and for one instance the batch decode, and their registers (the
+// results are those of the general kernels, which serve every other run).
 template <class F, int Dm, bool TGm = false, int LEANm = 0>
 struct PD : F {
   static constexpr int D = Dm;
   static constexpr bool TG = TGm;
   static constexpr bool LEAN = LEANm != 0;
-  static constexpr bool SINGLE = LEANm == 1;  // one instance, known at compile time
+  static constexpr bool SINGLE = LEANm == 1 || LEANm == 3;  // one instance, known at compile time
+  static constexpr bool STATIC = LEANm == 1 || LEANm == 2;  // no components
 };
 using P64 = PD<F64, 1>;
 using P32 = PD<F32, 1>;
@@ -160,6 +171,21 @@ using P32G = PD<F32, 1, true>;
 using P32L = PD<F32, 1, false, 1>;
 using P32LB = PD<F32, 1, false, 2>;
 using P32GL = PD<F32, 1, true, 2>;  // tangent mode, static potential, no event log
+using P32T = PD<F32, 1, false, 3>;  // components, no event log (one-launch periods only)
+using P64L = PD<F64, 1, false, 2>;  // FP64, static, no event log (one-launch periods only)
+
+// The model whose kernel runs a driver's periods as one launch (k_period),
+// void if none does: the lean models and the FP32 4D one themselves, and for
+// the general FP32 and FP64 models, in contexts without an event log, the
+// models above.
+template <class P>
+struct FusedModel { using type = void; };
+template <> struct FusedModel<P32L> { using type = P32L; };
+template <> struct FusedModel<P32LB> { using type = P32LB; };
+template <> struct FusedModel<P32GL> { using type = P32GL; };
+template <> struct FusedModel<Q32> { using type = Q32; };
+template <> struct FusedModel<P32> { using type = P32T; };
+template <> struct FusedModel<P64> { using type = P64L; };
 
 // Resident 256-thread blocks per SM a queue kernel is built for (its launch
 // bound).  The lean FP32 kernels and the FP32 4D kernels fit 64 registers,
@@ -180,11 +206,6 @@ __host__ __device__ constexpr int max_blocks_model() {
 template <class P>
 __host__ __device__ constexpr bool inline_drain() {
   return !P::is64 && (P::LEAN || (P::D == 2 && !P::TG));
-}
-// ... and run a regenerating period as one launch (k_period).
-template <class P>
-__host__ __device__ constexpr bool fused_period() {
-  return inline_drain<P>();
 }
 static_assert(max_blocks_model<P32L>() <= kMaxBlocksPerSm, "tuning range");
 
@@ -231,7 +252,7 @@ struct SEntry;
 template <class T>
 struct Inst {
   T gamma0, cacc, sig_k, xc;  // rate, acceptance factor C/(2 gamma0), kick scale, centre
-  double p_hi;                // FP64: u0 < p_hi may start an event in an interval
+  unsigned long long n_hi;    // FP64: n53 < n_hi (u0 < p_hi) may start an event in an interval
   float p_any_f;              // FP32: P(candidate) per interval
   float ilq;                  // FP32: 1 / ln(1 - p_any), the geometric gap's scale
   float ig0;                  // FP32: 1 / gamma0
@@ -588,9 +609,28 @@ struct Draw<P, true> {
   __device__ static double first(const KP<P>& p, const Inst<double>& ip,
                                  unsigned long long pid, int l, double to, bool /*root*/,
                                  State&) {
+    return P::add(to, life(ip, first_n(p, pid, l)));
+  }
+  __device__ static unsigned long long first_n(const KP<P>& p, unsigned long long pid, int l) {
     const uint4 r = philox_ks(p.ks, (uint32_t)pid, (uint32_t)(pid >> 32), (uint32_t)l, 0u);
-    const double u0 = u53(r.x, r.y);
-    return P::add(to, P::div(-log1p(-u0), ip.gamma0));
+    return n53(r.x, r.y);
+  }
+  // the life-length -log1p(-u)/gamma0 of the uniform n 2^-53
+  __device__ static double life(const Inst<double>& ip, unsigned long long n) {
+    return __ddiv_rn(-log1p(-u53_of(n)), ip.gamma0);
+  }
+  // event j, up to the uniform (as its 53-bit integer) of the gap to the
+  // next event: event() and event4() below turn it into the gap
+  __device__ static void event_n(const KP<P>& p, unsigned long long pid, int l, unsigned j,
+                                 double& z, double& u3, unsigned long long& n4) {
+    const uint32_t lo = (uint32_t)pid, hi = (uint32_t)(pid >> 32);
+    const uint4 a = philox_ks(p.ks, lo, hi, (uint32_t)l, 1u + 2u * j);
+    const uint4 b = philox_ks(p.ks, lo, hi, (uint32_t)l, 2u + 2u * j);
+    const double u1 = u53(a.x, a.y), u2 = u53(a.z, a.w);
+    u3 = u53(b.x, b.y);
+    n4 = n53(b.z, b.w);
+    z = __dmul_rn(__dsqrt_rn(__dmul_rn(-2.0, log1p(-u1))),
+                  cos(__dmul_rn(6.283185307179586476925286766559, u2)));
   }
   __device__ static bool event4(const KP<P>& p, const Inst<double>& ip, unsigned long long pid,
                                 int l, unsigned j, const PV<P>& xe, const State&, int& comp,
@@ -609,15 +649,9 @@ struct Draw<P, true> {
   __device__ static void event(const KP<P>& p, const Inst<double>& ip, unsigned long long pid,
                                int l, unsigned j, bool /*root*/, const State&, double& z,
                                double& u3, double& gap) {
-    const uint32_t lo = (uint32_t)pid, hi = (uint32_t)(pid >> 32);
-    const uint4 a = philox_ks(p.ks, lo, hi, (uint32_t)l, 1u + 2u * j);
-    const uint4 b = philox_ks(p.ks, lo, hi, (uint32_t)l, 2u + 2u * j);
-    const double u1 = u53(a.x, a.y), u2 = u53(a.z, a.w);
-    u3 = u53(b.x, b.y);
-    const double u4 = u53(b.z, b.w);
-    z = __dmul_rn(__dsqrt_rn(__dmul_rn(-2.0, log1p(-u1))),
-                  cos(__dmul_rn(6.283185307179586476925286766559, u2)));
-    gap = __ddiv_rn(-log1p(-u4), ip.gamma0);
+    unsigned long long n4;
+    event_n(p, pid, l, j, z, u3, n4);
+    gap = life(ip, n4);
   }
 };
 
@@ -830,6 +864,19 @@ static_assert(sizeof(SEntry<P32L>) == 64 && sizeof(SEntry<P32LB>) == 64, "SEntry
 static_assert(sizeof(SEntry<Q32>) == 64, "SEntry layout");
 static_assert(sizeof(SEntry<P32G>) == 64, "SEntry layout");
 
+// A deferred segment of a one-launch FP64 period: t is the time of its last
+// event (or its birth) and n the uniform of the life-length that follows,
+// whose logarithm is only taken when the segment is.
+template <class P>
+struct DEntry : TanOf<P> {
+  unsigned long long pid, n;
+  PV<P> xo, k;
+  double to, w, t;
+  int l;
+  unsigned j;   // as SEntry's
+};
+static_assert(sizeof(DEntry<P64L>) <= sizeof(SEntry<P64L>), "DEntry fits SEntry's segments");
+
 constexpr unsigned kRootFlag = 0x80000000u;
 
 // FP32 candidate clock.  Whether an interval holds a candidate is a
@@ -1021,15 +1068,15 @@ struct alignas(P::TG ? 8 : 16) Birth : TanOf<P> {
 // table_kick; the pair is k +/- kappa e_m with e_0 = (1, 0), e_1 = (0, 1),
 // e_2 = (1, -1).  Returns whether a pair is made (its data in b) and sets
 // the gap to the segment's next event.
-template <class P>
+// In a one-launch FP64 period Next is the gap's uniform as an integer.
+template <class P, class Next>
 __device__ __forceinline__ bool event_decide(const KP<P>& p, const Inst<typename P::T>& ip,
                                              int inst, unsigned long long pid,
                                              const PV<P>& xo, typename P::T to,
                                              const PV<P>& k, typename P::T w,
                                              const typename Draw<P>::State& st, int l,
                                              unsigned j, bool root, typename P::T t,
-                                             const TanOf<P>& tau, Birth<P>& b,
-                                             typename P::T& gap) {
+                                             const TanOf<P>& tau, Birth<P>& b, Next& gap) {
   using T = typename P::T;
   const PV<P> xe = pos_at(p, xo, to, k, t);
   T kap, fac;
@@ -1039,8 +1086,9 @@ __device__ __forceinline__ bool event_decide(const KP<P>& p, const Inst<typename
   if constexpr (P::D == 1) {
     T z, sg, u3;
     bool flip;
-    Draw<P>::event(p, ip, pid, l, j, root, st, z, u3, gap);
-    if (P::LEAN || p.ncomp == 0) {  // the static barrier: kick, |sin| ratio, orientation
+    if constexpr (std::is_same_v<Next, T>) Draw<P>::event(p, ip, pid, l, j, root, st, z, u3, gap);
+    else Draw<P>::event_n(p, pid, l, j, z, u3, gap);
+    if (P::STATIC || (!P::LEAN && p.ncomp == 0)) {  // the static barrier: kick, |sin| ratio, orientation
       kap = P::mul(ip.sig_k, z);
       sg = P::sn(P::mul(P::mul((T)2, P::sub(xe.c[0], ip.xc)), kap));
       fac = P::mul(ip.cacc, (T)fabs(sg));
@@ -1088,14 +1136,13 @@ __device__ __forceinline__ bool event_decide(const KP<P>& p, const Inst<typename
 }
 
 // The pair of an accepted event (Alg. 1 item 3): ids, kills outside the
-// k-range, tallies, the event log, then each offspring settled or, when it
-// has an event of its own in the interval, handed to `later`.
-template <class P, int DST, class Later>
-__device__ __forceinline__ void event_pair(const KP<P>& p, const Inst<typename P::T>& ip,
-                                           WarpCounts& wc, Acc& acc, const Birth<P>& b,
-                                           Later later) {
+// k-range, tallies, the event log, then child(id, wavevector, weight, tangent
+// weight) for each offspring that is not killed.
+template <class P, class Child>
+__device__ __forceinline__ void pair_of(const KP<P>& p, const Inst<typename P::T>& ip, Acc& acc,
+                                        const Birth<P>& b, Child child) {
   using T = typename P::T;
-  const int l = ent_l(b.l), inst = ent_inst(b.l);
+  const int l = ent_l(b.l);
   const uint4 h = philox_ks(p.ks, (uint32_t)b.pid, (uint32_t)(b.pid >> 32), (uint32_t)l,
                             kDrawPids | b.j);
   const unsigned long long pid_p = (1ull << 63) | ((((unsigned long long)h.y << 32) | h.x) >> 1);
@@ -1139,22 +1186,37 @@ __device__ __forceinline__ void event_pair(const KP<P>& p, const Inst<typename P
 #pragma unroll
   for (int c = 0; c < 2; ++c) {
     if (c == 0 ? kill_p : kill_m) continue;
-    SEntry<P> ch;
+    TanOf<P> tau;
     if constexpr (P::TG) {
-      ch.th = c == 0 ? tp.th : -tp.th;
-      ch.tw = c == 0 ? tp.tw : -tp.tw;
+      tau.th = c == 0 ? tp.th : -tp.th;
+      tau.tw = c == 0 ? tp.tw : -tp.tw;
     }
-    ch.pid = c == 0 ? pid_p : pid_m;
+    child(c == 0 ? pid_p : pid_m, c == 0 ? b.kp : b.km, c == 0 ? wc_ : -wc_, tau);
+  }
+}
+
+// Each offspring settled or, when it has an event of its own in the
+// interval, handed to `later`.
+template <class P, int DST, class Later>
+__device__ __forceinline__ void event_pair(const KP<P>& p, const Inst<typename P::T>& ip,
+                                           WarpCounts& wc, Acc& acc, const Birth<P>& b,
+                                           Later later) {
+  using T = typename P::T;
+  const int l = ent_l(b.l), inst = ent_inst(b.l);
+  pair_of<P>(p, ip, acc, b, [&](unsigned long long pid, const PV<P>& k, T w, const TanOf<P>& tau) {
+    SEntry<P> ch;
+    static_cast<TanOf<P>&>(ch) = tau;
+    ch.pid = pid;
     ch.xo = b.xe;
     ch.to = b.t;
-    ch.k = c == 0 ? b.kp : b.km;
-    ch.w = c == 0 ? wc_ : -wc_;
+    ch.k = k;
+    ch.w = w;
     ch.l = b.l;
     ch.j = 0;
     ch.t = Draw<P>::first(p, ip, ch.pid, l, b.t, false, ch.st);
     if (ch.t < p.dt) later(ch);
     else settle<P, DST>(p, wc, acc, inst, ch.pid, ch.xo, ch.to, ch.k, ch.w, l, ch, ch.t);
-  }
+  });
 }
 
 // Event j of a segment at time t: the decision and, when a pair is made,
@@ -1236,45 +1298,72 @@ __device__ __forceinline__ int base_instance(const KP<P>& p, unsigned long long 
   return lo;
 }
 
-// Append one candidate entry per flagged lane (interval c, the position
-// streamed from the lane's interval ls to c) to the warp's segment eq_seg
-// of the candidate queue (null when the warp owns none); ecount is the
-// segment's count, held in a register by every lane.  Every lane of the
-// warp calls it.
+// Where a warp's candidate intervals go, by their number in its list: the
+// warp's segment of a round's queue (null when the warp owns none) ...
 template <class P>
-__device__ __forceinline__ void append_candidate(const KP<P>& p, unsigned& ecount,
-                                                 FEntry<P>* eq_seg, bool has,
-                                                 unsigned long long pid, const PV<P>& x,
+struct CandSegment {
+  static constexpr bool STACK = false;
+  FEntry<P>* seg;
+  unsigned cap;
+  __device__ __forceinline__ bool put(unsigned q, const FEntry<P>& e) const {
+    if (!seg || q >= cap) return false;
+    seg[q] = e;
+    return true;
+  }
+};
+
+// ... or (FP64 one-launch periods) the warp's stack: kEStack entries in
+// shared memory, the rest in the segment.
+constexpr unsigned kEStack = 128;
+template <class P>
+struct CandStack {
+  static constexpr bool STACK = true;
+  FEntry<P>* top;
+  FEntry<P>* seg;
+  unsigned cap;   // of both
+  __device__ __forceinline__ bool put(unsigned q, const FEntry<P>& e) const {
+    if (q >= cap) return false;
+    if (q < kEStack) top[q] = e;
+    else seg[q - kEStack] = e;
+    return true;
+  }
+  __device__ __forceinline__ FEntry<P> get(unsigned q) const {
+    return q < kEStack ? top[q] : seg[q - kEStack];
+  }
+};
+
+// Append one candidate entry per flagged lane (interval c, the position
+// streamed from the lane's interval ls to c) to the warp's candidates;
+// ecount is their count, held in a register by every lane.  Every lane of
+// the warp calls it.
+template <class P, class Q>
+__device__ __forceinline__ void append_candidate(const KP<P>& p, unsigned& ecount, const Q& cq,
+                                                 bool has, unsigned long long pid, const PV<P>& x,
                                                  const PV<P>& k, typename P::T w, int ls, int c,
                                                  int inst, const TanOf<P>& tau) {
   const int lane = threadIdx.x & 31;
   const unsigned bal = __ballot_sync(kFull, has);
   if (has) {
     const unsigned q = ecount + __popc(bal & ((1u << lane) - 1u));
-    if (eq_seg && q < p.eseg) {
-      FEntry<P> e;
-      static_cast<TanOf<P>&>(e) = tau;
-      e.pid = pid;
+    FEntry<P> e;
+    static_cast<TanOf<P>&>(e) = tau;
+    e.pid = pid;
 #pragma unroll
-      for (int d = 0; d < P::D; ++d) e.x.c[d] = stream_n<P>(x.c[d], k.c[d], p.dtv, c - ls);
-      e.k = k;
-      e.w = w;
-      e.l = ent_pack(c, inst);
-      eq_seg[q] = e;
-    } else {
-      set_err(p.cnt, ERR_CAP_EQUEUE);
-    }
+    for (int d = 0; d < P::D; ++d) e.x.c[d] = stream_n<P>(x.c[d], k.c[d], p.dtv, c - ls);
+    e.k = k;
+    e.w = w;
+    e.l = ent_pack(c, inst);
+    if (!cq.put(q, e)) set_err(p.cnt, ERR_CAP_EQUEUE);
   }
   ecount += __popc(bal);
 }
 
-template <class P, int SRC, int DST>
+template <class P, int SRC, int DST, class Q>
 __device__ __forceinline__ void flight_tile(const KP<P>& p, WarpCounts& wc, Acc& acc, bool act,
                                             unsigned long long slot, PV<P> x, const PV<P>& k,
                                             typename P::T w, unsigned long long pid, int ls,
                                             int inst, const TanOf<P>& tau,
-                                            uint32_t gbits, unsigned& ecount,
-                                            FEntry<P>* eq_seg) {
+                                            uint32_t gbits, unsigned& ecount, const Q& cq) {
   using T = typename P::T;
   const int lane = threadIdx.x & 31;
   const unsigned g = global_warp();
@@ -1285,11 +1374,22 @@ __device__ __forceinline__ void flight_tile(const KP<P>& p, WarpCounts& wc, Acc&
   // event.  Bit b of mask is interval l0 + b.
   unsigned mask = 0;
   const uint32_t plo = (uint32_t)pid, phi = (uint32_t)(pid >> 32);
-  if (act) {
+  if constexpr (P::is64 && Q::STACK) {
+    // FP64 in a one-launch period: interval by interval, each candidate
+    // written where the particle is when its interval begins
+    for (int l = p.l0; l < p.L; ++l) {
+      const bool has = act && Draw<P>::first_n(p, pid, l) < ip.n_hi;
+      if (__ballot_sync(kFull, has))
+        append_candidate<P>(p, ecount, cq, has, pid, x, k, w, l, l, inst, tau);
+#pragma unroll
+      for (int d = 0; d < P::D; ++d) x.c[d] = P::stream(x.c[d], k.c[d], p.dtv);
+    }
+    if (act) acc.psteps += (unsigned)p.len;
+  } else if (act) {
     if constexpr (P::is64) {
       for (int l = ls; l < p.L; ++l) {
         const uint4 r = philox_ks(p.ks, plo, phi, (uint32_t)l, 0u);
-        if (u53(r.x, r.y) < ip.p_hi) mask |= 1u << (l - p.l0);
+        if (n53(r.x, r.y) < ip.n_hi) mask |= 1u << (l - p.l0);
       }
     } else if (ls < p.L) {
       // FP32: the first candidate interval from ls on, a geometric gap from
@@ -1308,6 +1408,7 @@ __device__ __forceinline__ void flight_tile(const KP<P>& p, WarpCounts& wc, Acc&
     acc.psteps += (unsigned)(p.L - ls);
   }
 
+  if constexpr (!(P::is64 && Q::STACK)) {
   // ---- the warp's candidate entries.  Entry j of the warp (lanes in
   // order, intervals in order within a lane) goes to queue slot ecount + j and
   // is written by lane j mod 32, which fetches its owner's state with
@@ -1315,7 +1416,7 @@ __device__ __forceinline__ void flight_tile(const KP<P>& p, WarpCounts& wc, Acc&
   if constexpr (!P::is64) {
     // FP32: at most one entry per lane (the first candidate interval)
     if (__ballot_sync(kFull, mask != 0u))
-      append_candidate<P>(p, ecount, eq_seg, mask != 0u, pid, x, k, w, ls,
+      append_candidate<P>(p, ecount, cq, mask != 0u, pid, x, k, w, ls,
                           p.l0 + __ffs(mask) - 1, inst, tau);
   } else {
   const unsigned cnt = __popc(mask);
@@ -1357,20 +1458,16 @@ __device__ __forceinline__ void flight_tile(const KP<P>& p, WarpCounts& wc, Acc&
       if (j < total) {
         for (unsigned t = j - eo; t; --t) mo &= mo - 1;  // the (j - eo)-th set bit
         const int l = p.l0 + __ffs(mo) - 1;
-        const unsigned long long q = (unsigned long long)ecount + j;
-        if (eq_seg && q < p.eseg) {
-          FEntry<P> e;
-          static_cast<TanOf<P>&>(e) = to;
-          e.pid = po;
+        const unsigned q = ecount + j;
+        FEntry<P> e;
+        static_cast<TanOf<P>&>(e) = to;
+        e.pid = po;
 #pragma unroll
-          for (int d = 0; d < P::D; ++d) e.x.c[d] = stream_n<P>(xo.c[d], ko.c[d], p.dtv, l - lo_s);
-          e.k = ko;
-          e.w = wo;
-          e.l = ent_pack(l, io);
-          eq_seg[q] = e;
-        } else {
-          set_err(p.cnt, ERR_CAP_EQUEUE);
-        }
+        for (int d = 0; d < P::D; ++d) e.x.c[d] = stream_n<P>(xo.c[d], ko.c[d], p.dtv, l - lo_s);
+        e.k = ko;
+        e.w = wo;
+        e.l = ent_pack(l, io);
+        if (!cq.put(q, e)) set_err(p.cnt, ERR_CAP_EQUEUE);
       }
     }
     ecount += total;
@@ -1381,6 +1478,7 @@ __device__ __forceinline__ void flight_tile(const KP<P>& p, WarpCounts& wc, Acc&
   if (act) {
 #pragma unroll
     for (int d = 0; d < P::D; ++d) x.c[d] = stream_n<P>(x.c[d], k.c[d], p.dtv, p.L - ls);
+  }
   }
 
   // ---- the particle's own final state ----------------------------------
@@ -1525,12 +1623,35 @@ __device__ __forceinline__ void flight_tile(const KP<P>& p, WarpCounts& wc, Acc&
 
 }
 
-// The work of one flight launch for the calling warp: its share of the
-// source's particles carried through [ls, L) into the sink, their candidate
-// intervals appended to the warp's candidate segment (ecount entries so far).
-template <class P, int SRC, int DST>
+// What a flight reads of its source, once per kernel.
+template <int SRC>
+struct SourceInfo {
+  unsigned long long n = 0, n_base = 0, base_pid = 0;
+  unsigned nz = 0;
+  template <class P>
+  __device__ __forceinline__ void load(const KP<P>& p) {
+    if constexpr (SRC == SRC_ARRAY) {
+      n = p.cnt->n_src;
+      n_base = p.cnt->n_base;
+      base_pid = p.cnt->base_pid;
+    } else if constexpr (SRC == SRC_REGEN || SRC == SRC_TREGEN) {
+      n = min(SRC == SRC_TREGEN ? p.cnt->tan_total : p.cnt->regen_total,
+              (unsigned long long)p.tile_cap * 32ull);
+      nz = (unsigned)(SRC == SRC_TREGEN ? p.cnt->tan_nz : p.cnt->nz_count);
+    }
+  }
+};
+
+// The work of a flight for the calling warp: its share of the source's
+// particles, from slot `next` on, carried through [ls, L) into the sink,
+// their candidate intervals appended to the warp's (ecount so far); with a
+// stack, until that holds at least `fill`.  Leaves `next` at the first slot
+// not taken.
+template <class P, int SRC, int DST, class Q>
 __device__ __forceinline__ void flight_body(const KP<P>& p, WarpCounts& wc, Acc& acc,
-                                            unsigned& ecount, FEntry<P>* const eq_seg) {
+                                            const SourceInfo<SRC>& info, unsigned& ecount,
+                                            const Q& cq, unsigned long long& next,
+                                            unsigned fill = ~0u) {
   using T = typename P::T;
   const int lane = threadIdx.x & 31;
   const unsigned g = global_warp();
@@ -1553,7 +1674,7 @@ __device__ __forceinline__ void flight_body(const KP<P>& p, WarpCounts& wc, Acc&
         nx = nx2;
         nx2 = i + 64 < n ? seg[i + 64] : none;
         flight_tile<P, SRC, DST>(p, wc, acc, act, 0, e.x, e.k, e.w, e.pid, ent_l(e.l),
-                                 ent_inst(e.l), e, 0u, ecount, eq_seg);
+                                 ent_inst(e.l), e, 0u, ecount, cq);
       }
     }
   } else {
@@ -1565,28 +1686,24 @@ __device__ __forceinline__ void flight_body(const KP<P>& p, WarpCounts& wc, Acc&
     const uint32_t* nz_cell = TR ? p.tnz_cell : p.nz_cell;
     const unsigned long long* nz_start = TR ? p.tnz_start : p.nz_start;
     const unsigned long long* islot = TR ? p.tinst_slot : p.inst_slot;
-    unsigned long long n;
-    if constexpr (SRC == SRC_ARRAY) n = p.cnt->n_src;
-    else n = min(TR ? p.cnt->tan_total : p.cnt->regen_total, (unsigned long long)p.tile_cap * 32ull);
-    const unsigned long long n_base = p.cnt->n_base, base_pid = p.cnt->base_pid;
+    [[maybe_unused]] const unsigned long long n_base = info.n_base, base_pid = info.base_pid;
     // slots and plan positions of a regeneration index in 32 bits (the
     // capacity is below 2^32 - 2^20, so no sum below overflows)
     using IX = std::conditional_t<RG, unsigned, unsigned long long>;
-    const IX nn = (IX)n;
-    const IX nz = RG ? (IX)(TR ? p.cnt->tan_nz : p.cnt->nz_count) : (IX)0;
+    const IX nn = (IX)info.n, first = (IX)next;
+    [[maybe_unused]] const IX nz = (IX)info.nz;
     // regeneration plan entries, loaded ahead: the first nonzero cell a0 two
     // tiles ahead, the starts and cells one tile ahead
     const IX stride = (IX)(nwarps * 32ull);
     IX a0_next = 0, idx_n = 0, st_n = (IX)~0ull;
     uint32_t cw_n = 0u;
     if constexpr (RG) {
-      const IX b0 = (IX)(g * 32ull);
-      if (b0 < nn) {
-        idx_n = tile_nz[b0 >> 5] + lane;
+      if (first < nn) {
+        idx_n = tile_nz[first >> 5] + lane;
         st_n = idx_n < nz ? (IX)nz_start[idx_n] : (IX)~0ull;
         cw_n = idx_n < nz ? nz_cell[idx_n] : 0u;
       }
-      if (b0 + stride < nn) a0_next = tile_nz[(b0 + stride) >> 5];
+      if (first + stride < nn) a0_next = tile_nz[(first + stride) >> 5];
     }
     // one tile of 32 slots; a full tile (every tile but a warp's last) is
     // compiled apart with every lane active, which drops the per-lane
@@ -1596,7 +1713,7 @@ __device__ __forceinline__ void flight_body(const KP<P>& p, WarpCounts& wc, Acc&
     constexpr bool PIPE = P::SINGLE && SRC == SRC_REGEN;
     uint4 r_next = make_uint4(0u, 0u, 0u, 0u);
     if constexpr (PIPE) {
-      const unsigned long long q0 = p.regen_base | (unsigned long long)((IX)(g * 32ull) + lane);
+      const unsigned long long q0 = p.regen_base | (unsigned long long)(first + (IX)lane);
       r_next = philox_ks(p.ks, (uint32_t)q0, (uint32_t)(q0 >> 32), kStepRegen, 0u);
     }
     auto tile = [&](const IX base, auto full) {
@@ -1716,12 +1833,14 @@ __device__ __forceinline__ void flight_body(const KP<P>& p, WarpCounts& wc, Acc&
         }
       }
       flight_tile<P, SRC, DST>(p, wc, acc, act, slot, x, k, w, pid, act ? p.l0 : p.L, inst, tau,
-                               gbits, ecount, eq_seg);
+                               gbits, ecount, cq);
     };
-    for (IX base = (IX)(g * 32ull); base < nn; base += stride) {
+    IX base = first;
+    for (; base < nn && (!Q::STACK || ecount < fill); base += stride) {
       if (base + (IX)32 <= nn) tile(base, std::true_type{});
       else tile(base, std::false_type{});
     }
+    next = base;
   }
 
 }
@@ -1739,8 +1858,11 @@ __global__ void __launch_bounds__(kBlock, (max_blocks<P, DST>())) k_flight(const
   const unsigned g = global_warp();
   // the warp's candidate segment and its count, in registers
   unsigned ecount = wc.e;
-  FEntry<P>* const eq_seg = g < (unsigned)p.nseg ? p.eq + (long long)g * p.eseg : nullptr;
-  flight_body<P, SRC, DST>(p, wc, acc, ecount, eq_seg);
+  const CandSegment<P> cq{g < (unsigned)p.nseg ? p.eq + (long long)g * p.eseg : nullptr, p.eseg};
+  SourceInfo<SRC> info;
+  info.load(p);
+  unsigned long long next = g * 32ull;
+  flight_body<P, SRC, DST>(p, wc, acc, info, ecount, cq, next);
   if (lane == 0) wc.e = ecount;
   store_counts(p, wc, 0, false, true, DST == DST_BIN2);
   block_reduce_add(red, acc.psteps, &p.cnt->ledger[SRC == SRC_QUEUE ? LG_PSTEPS : LG_PSTEPS0]);
@@ -1795,133 +1917,6 @@ __device__ __forceinline__ void copy_entry_async(FEntry<P>* dst, const FEntry<P>
 #pragma unroll
   for (unsigned w = 0; w < sizeof(FEntry<P>) / 8; ++w)
     cp_async8((char*)dst + 8 * w, (const char*)src + 8 * w);
-}
-
-// One round of the event kernel for the calling warp: the first event of
-// each candidate interval in seg[0, n) (one per lane), the pairs, and, in the
-// kernels that finish them themselves, every deferred segment; the pairs of
-// first events are added to first_pairs.  stage and buf are the warp's
-// shared staging tiles and accepted-event buffer.
-template <class P, int DST>
-__device__ __forceinline__ void event_round(const KP<P>& p, WarpCounts& wc, Acc& acc,
-                                            const FEntry<P>* seg, unsigned n,
-                                            FEntry<P> (*stage)[32], Birth<P>* buf,
-                                            unsigned& first_pairs) {
-  using T = typename P::T;
-  const int lane = threadIdx.x & 31;
-  const unsigned g = global_warp();
-  auto later = [&](const SEntry<P>& ch) { defer<P>(p, wc, 1, ch); };
-  // FP32 2D: the accepted events of the warp's tiles wait in a per-warp
-  // buffer and their pairs are made 32 at a time, so that every lane has one
-  // (the acceptance would otherwise leave a third of the lanes idle there);
-  // the 4D events, with larger records and more registers, measured slower so
-  constexpr bool CMP = !P::is64 && P::D == 1;
-  unsigned nb = 0;  // births in the buffer (the same in every lane)
-  auto make_pairs = [&](unsigned lim) {
-    while (nb >= lim) {
-      const unsigned take = min(nb, 32u);
-      __syncwarp();
-      if ((unsigned)lane < take) {
-        const Birth<P> bb = buf[nb - take + lane];
-        event_pair<P, DST>(p, inst_of(p, ent_inst(bb.l)), wc, acc, bb, later);
-      }
-      __syncwarp();
-      nb -= take;
-    }
-  };
-  const unsigned events0 = acc.events;
-  // each lane copies its entry of the next tile into shared memory
-  // asynchronously while the current tile is processed
-  if ((unsigned)lane < n) copy_entry_async<P>(&stage[0][lane], seg + lane);
-  cp_async_commit();
-  unsigned t = 0;
-  for (unsigned b = 0; b < n; b += 32, ++t) {
-    const unsigned i = b + lane;
-    if (i + 32 < n) copy_entry_async<P>(&stage[(t + 1) & 1][lane], seg + i + 32);
-    cp_async_commit();
-    cp_async_wait<1>();
-    FEntry<P> e{};
-    if (i < n) e = stage[t & 1][lane];
-    bool made = false;
-    Birth<P> bb;
-    if (i < n) {
-      const int l = ent_l(e.l), inst = ent_inst(e.l);
-      const Inst<T> ip = inst_of(p, inst);
-      SEntry<P> s;
-      static_cast<TanOf<P>&>(s) = static_cast<const TanOf<P>&>(e);
-      s.pid = e.pid;
-      s.xo = e.x;
-      s.to = (T)0;
-      s.k = e.k;
-      s.w = e.w;
-      s.l = e.l;
-      s.t = Draw<P>::first(p, ip, e.pid, l, (T)0, true, s.st);
-      if (s.t < p.dt) {
-        ++acc.cand;
-        T gap;
-        if constexpr (CMP) {
-          made = event_decide<P>(p, ip, inst, s.pid, s.xo, s.to, s.k, s.w, s.st, l, 0u, true,
-                                 s.t, s, bb, gap);
-        } else {
-          gap = do_event<P, DST>(p, ip, inst, wc, acc, s.pid, s.xo, s.to, s.k, s.w, s.st, l,
-                                 0u, true, s.t, later, s);
-        }
-        s.t = P::add(s.t, gap);
-        if (s.t < p.dt) {
-          s.j = 1u | kRootFlag;
-          defer<P>(p, wc, 1, s);
-        } else {
-          chain_next<P>(p, wc, s);
-        }
-      }
-    }
-    if constexpr (CMP) {
-      const unsigned bal = __ballot_sync(kFull, made);
-      if (made) buf[nb + __popc(bal & ((1u << lane) - 1u))] = bb;
-      nb += __popc(bal);
-      make_pairs(32u);
-    }
-  }
-  cp_async_wait<0>();
-  if constexpr (CMP) make_pairs(1u);
-  // so far the warp has made only first events' pairs
-  first_pairs += acc.events - events0;
-  if constexpr (inline_drain<P>()) {
-    // These kernels finish their warp's deferred segments here instead of
-    // in launches of their own: one event per lane per pass (Alg. 1 item 3,
-    // offspring born inside the interval included), a segment with another
-    // event in its interval appended again to the same list, until the list
-    // is used up.  Its count is then zero for the launches that follow.
-    const SEntry<P>* dl = p.dq[1] + (size_t)g * p.dseg;
-    unsigned rd = 0;
-    for (;;) {
-      __syncwarp();
-      const unsigned end = min(wc.d, p.dseg);
-      if (rd >= end || g >= (unsigned)p.nseg) break;
-      const unsigned i = rd + lane;
-      if (i < end) {
-        SEntry<P> s = dl[i];
-        const unsigned j = s.j & ~kRootFlag;
-        const int l = ent_l(s.l), inst = ent_inst(s.l);
-        const Inst<T> ip = inst_of(p, inst);
-        const T gap = do_event<P, DST>(p, ip, inst, wc, acc, s.pid, s.xo, s.to, s.k, s.w, s.st,
-                                       l, j, (s.j & kRootFlag) != 0u, s.t, later, s);
-        s.t = P::add(s.t, gap);
-        if (s.t < p.dt) {
-          s.j = (j + 1) | (s.j & kRootFlag);
-          defer<P>(p, wc, 1, s);
-        } else if (!(s.j & kRootFlag)) {
-          settle<P, DST>(p, wc, acc, inst, s.pid, s.xo, s.to, s.k, s.w, l, s, s.t);
-        } else {
-          chain_next<P>(p, wc, s);
-        }
-      }
-      rd = min(rd + 32u, end);
-    }
-    __syncwarp();
-    if (lane == 0) wc.d = 0;
-    __syncwarp();
-  }
 }
 
 template <class P, int DST>
@@ -2074,44 +2069,185 @@ __global__ void __launch_bounds__(kBlock, (max_blocks<P, DST>())) k_event(const 
   reduce_event_tallies(red, acc, p.cnt, DST == DST_BIN2);
 }
 
-// A whole resampling period in one launch (the lean models): each warp
-// runs its share of the first wave (in the tangent mode, then its share of
-// the tangent particles' first wave), then the event rounds over its own
-// candidate segments.  Warp g writes candidate segment g and only warp g
-// reads it, in this launch as in the launch-per-round schedule, so the
-// rounds need no barrier between warps: a warp starts its next round as
-// soon as it has finished the previous one, and the warps of an SM mix the
-// two phases.  Round r appends to the candidate buffer round r reads not
-// (p.eq and p.eq_alt alternate); the deferred segments are finished inside
-// each round.  Results are those of the launch-per-round schedule, bit for
-// bit (every draw is keyed by particle and interval).
+constexpr unsigned kBirths = 64;      // accepted events a warp may hold
+constexpr int kPeriodBlocks = 3;      // resident blocks per SM k_period is built for
+
+// Dynamic shared memory of a warp in k_period: FP64, the top of its candidate
+// stack and its accepted events.
+template <class P>
+__host__ __device__ constexpr size_t period_warp_bytes() {
+  return P::is64 ? kEStack * sizeof(FEntry<P>) + kBirths * sizeof(Birth<P>) : 0;
+}
+
+// A whole flight of a chunk in one launch: each warp carries its share of
+// the source (and in the tangent mode, of the tangent particles) to the
+// sink, then every event of their candidate intervals and all their
+// offspring.  Warp g writes candidate and deferred segment g and only warp g
+// reads them, so there is no barrier between warps: each goes on as soon as
+// it can, and the warps of an SM mix the phases.  Every draw is keyed by
+// particle and interval: the results are those of the launch-per-round
+// schedule, bit for bit.
+//
+// FP32 (period_fp32): the first wave, then rounds over the warp's candidates,
+// round r appending to the buffer round r reads not; each round finishes its
+// own accepted events and deferred segments.  Other schedules of the same
+// passes measured slower (1e8 particles, 3.12 ms so): the next 32 of any list
+// that holds 32, fresh particles only when none does, 3.82 ms (it costs the
+// read-ahead of plan and candidates); candidates through one ring 3.38 ms;
+// one loop body for first and deferred events 3.47 ms.
+// One round of the event kernel for the calling warp: the first event of
+// each candidate interval in seg[0, n) (one per lane), the pairs, and every
+// deferred segment; the pairs of
+// first events are added to first_pairs.  stage and buf are the warp's
+// shared staging tiles and accepted-event buffer.
 template <class P, int DST>
-__global__ void __launch_bounds__(kBlock, 3) k_period(const KP<P> p_) {
-  const KP<P> p = with_period(p_);
-  __shared__ unsigned long long red[kWarps];
-  __shared__ WarpCounts s_wc[kWarps];
+__device__ __forceinline__ void event_round(const KP<P>& p, WarpCounts& wc, Acc& acc,
+                                            const FEntry<P>* seg, unsigned n,
+                                            FEntry<P> (*stage)[32], Birth<P>* buf,
+                                            unsigned& first_pairs) {
+  using T = typename P::T;
   const int lane = threadIdx.x & 31;
-  WarpCounts& wc = s_wc[threadIdx.x >> 5];
-  Acc acc;
-  acc.zero();
-  load_counts(p, wc, 1);
+  const unsigned g = global_warp();
+  auto later = [&](const SEntry<P>& ch) { defer<P>(p, wc, 1, ch); };
+  // FP32 2D: the accepted events of the warp's tiles wait in a per-warp
+  // buffer and their pairs are made 32 at a time, so that every lane has one
+  // (the acceptance would otherwise leave a third of the lanes idle there);
+  // the 4D events, with larger records and more registers, measured slower so
+  constexpr bool CMP = !P::is64 && P::D == 1;
+  unsigned nb = 0;  // births in the buffer (the same in every lane)
+  auto make_pairs = [&](unsigned lim) {
+    while (nb >= lim) {
+      const unsigned take = min(nb, 32u);
+      __syncwarp();
+      if ((unsigned)lane < take) {
+        const Birth<P> bb = buf[nb - take + lane];
+        event_pair<P, DST>(p, inst_of(p, ent_inst(bb.l)), wc, acc, bb, later);
+      }
+      __syncwarp();
+      nb -= take;
+    }
+  };
+  const unsigned events0 = acc.events;
+  // each lane copies its entry of the next tile into shared memory
+  // asynchronously while the current tile is processed
+  if ((unsigned)lane < n) copy_entry_async<P>(&stage[0][lane], seg + lane);
+  cp_async_commit();
+  unsigned t = 0;
+  for (unsigned b = 0; b < n; b += 32, ++t) {
+    const unsigned i = b + lane;
+    if (i + 32 < n) copy_entry_async<P>(&stage[(t + 1) & 1][lane], seg + i + 32);
+    cp_async_commit();
+    cp_async_wait<1>();
+    FEntry<P> e{};
+    if (i < n) e = stage[t & 1][lane];
+    bool made = false;
+    Birth<P> bb;
+    if (i < n) {
+      const int l = ent_l(e.l), inst = ent_inst(e.l);
+      const Inst<T> ip = inst_of(p, inst);
+      SEntry<P> s;
+      static_cast<TanOf<P>&>(s) = static_cast<const TanOf<P>&>(e);
+      s.pid = e.pid;
+      s.xo = e.x;
+      s.to = (T)0;
+      s.k = e.k;
+      s.w = e.w;
+      s.l = e.l;
+      s.t = Draw<P>::first(p, ip, e.pid, l, (T)0, true, s.st);
+      if (s.t < p.dt) {
+        ++acc.cand;
+        T gap;
+        if constexpr (CMP) {
+          made = event_decide<P>(p, ip, inst, s.pid, s.xo, s.to, s.k, s.w, s.st, l, 0u, true,
+                                 s.t, s, bb, gap);
+        } else {
+          gap = do_event<P, DST>(p, ip, inst, wc, acc, s.pid, s.xo, s.to, s.k, s.w, s.st, l,
+                                 0u, true, s.t, later, s);
+        }
+        s.t = P::add(s.t, gap);
+        if (s.t < p.dt) {
+          s.j = 1u | kRootFlag;
+          defer<P>(p, wc, 1, s);
+        } else {
+          chain_next<P>(p, wc, s);
+        }
+      }
+    }
+    if constexpr (CMP) {
+      const unsigned bal = __ballot_sync(kFull, made);
+      if (made) buf[nb + __popc(bal & ((1u << lane) - 1u))] = bb;
+      nb += __popc(bal);
+      make_pairs(32u);
+    }
+  }
+  cp_async_wait<0>();
+  if constexpr (CMP) make_pairs(1u);
+  // so far the warp has made only first events' pairs
+  first_pairs += acc.events - events0;
+  {
+    // the warp's deferred segments: one event per lane per pass (Alg. 1 item
+    // 3, offspring born inside the interval included), a segment with another
+    // event in its interval appended again to the same list, until the list
+    // is used up
+    const SEntry<P>* dl = p.dq[1] + (size_t)g * p.dseg;
+    unsigned rd = 0;
+    for (;;) {
+      __syncwarp();
+      const unsigned end = min(wc.d, p.dseg);
+      if (rd >= end || g >= (unsigned)p.nseg) break;
+      const unsigned i = rd + lane;
+      if (i < end) {
+        SEntry<P> s = dl[i];
+        const unsigned j = s.j & ~kRootFlag;
+        const int l = ent_l(s.l), inst = ent_inst(s.l);
+        const Inst<T> ip = inst_of(p, inst);
+        const T gap = do_event<P, DST>(p, ip, inst, wc, acc, s.pid, s.xo, s.to, s.k, s.w, s.st,
+                                       l, j, (s.j & kRootFlag) != 0u, s.t, later, s);
+        s.t = P::add(s.t, gap);
+        if (s.t < p.dt) {
+          s.j = (j + 1) | (s.j & kRootFlag);
+          defer<P>(p, wc, 1, s);
+        } else if (!(s.j & kRootFlag)) {
+          settle<P, DST>(p, wc, acc, inst, s.pid, s.xo, s.to, s.k, s.w, l, s, s.t);
+        } else {
+          chain_next<P>(p, wc, s);
+        }
+      }
+      rd = min(rd + 32u, end);
+    }
+    __syncwarp();
+    if (lane == 0) wc.d = 0;
+    __syncwarp();
+  }
+}
+
+template <class P, int SRC, int DST>
+__device__ __forceinline__ void period_fp32(const KP<P>& p, WarpCounts& wc, Acc& acc,
+                                            unsigned& first_pairs, unsigned& psteps_first) {
+  const int lane = threadIdx.x & 31;
   const unsigned g = global_warp();
   const bool own = g < (unsigned)p.nseg;
   // the first wave: candidate intervals into buffer p.eq, segment g
-  unsigned ecount = wc.e;
-  flight_body<P, SRC_REGEN, DST>(p, wc, acc, ecount, own ? p.eq + (long long)g * p.eseg : nullptr);
-  if constexpr (P::TG) {  // the tangent particles of the same histogram join the first wave
-    flight_body<P, SRC_TREGEN, DST>(p, wc, acc, ecount,
-                                    own ? p.eq + (long long)g * p.eseg : nullptr);
+  unsigned ecount = 0;
+  {
+    const CandSegment<P> cq{own ? p.eq + (size_t)g * p.eseg : nullptr, p.eseg};
+    SourceInfo<SRC> src;
+    src.load(p);
+    unsigned long long next = g * 32ull;
+    flight_body<P, SRC, DST>(p, wc, acc, src, ecount, cq, next);
+    if constexpr (P::TG && SRC == SRC_REGEN) {  // the tangent particles of the same histogram
+      SourceInfo<SRC_TREGEN> tsrc;
+      tsrc.load(p);
+      next = g * 32ull;
+      flight_body<P, SRC_TREGEN, DST>(p, wc, acc, tsrc, ecount, cq, next);
+    }
   }
-  const unsigned psteps_first = acc.psteps;
-  constexpr bool CMP = !P::is64 && P::D == 1;
-  constexpr unsigned kBirths = 64;
+  psteps_first = acc.psteps;
+  constexpr bool CMP = P::D == 1;
   __shared__ Birth<P> s_birth[CMP ? kWarps : 1][CMP ? kBirths : 1];
   __shared__ __align__(16) FEntry<P> s_stage[kWarps][2][32];
-  static_assert(sizeof(s_birth) + sizeof(s_stage) + sizeof(s_wc) + sizeof(red) <= 48 * 1024,
+  static_assert(sizeof(s_birth) + sizeof(s_stage) + 512 <= 48 * 1024,
                 "a block declares at most 48 KB of static shared memory");
-  unsigned first_pairs = 0;
   unsigned n = own ? min(ecount, p.eseg) : 0u;
   for (int r = 0; r < p.len && n > 0u; ++r) {
     __syncwarp();
@@ -2126,12 +2262,212 @@ __global__ void __launch_bounds__(kBlock, 3) k_period(const KP<P> p_) {
     __syncwarp();
     n = min(wc.e, p.eseg);
   }
-  store_counts(p, wc, 1, false, false, DST == DST_BIN2);
+}
+
+// FP64 (period_fp64): FP64 instructions run at 1/64 of the FP32 rate here and
+// cost the same however few lanes are at work, so the lanes are kept filled
+// and the logarithms few:
+//   - the warp takes the next 32 of a list (candidates, deferred segments,
+//     accepted events) that holds 32, fresh particles only when none does, and
+//     part-filled lists only when its particles are used up;
+//   - an offspring (or a further event) that may fall into its interval, by
+//     the same integer comparison as the clock's, is deferred with its
+//     uniform, and the life-length's logarithm and division are taken when
+//     the segment is: nine of ten need none;
+//   - offspring fly on at once, and the candidate stack's top is in shared
+//     memory (depth first, it stays short).
+// An FP64 offspring's (or its last event's) end of interval l, in a
+// one-launch period: the flight through [l + 1, L) interval by interval (one
+// draw each, as flight_tile's clock), its candidates to `cand`, then the sink.
+template <class P, int DST, class Cand>
+__device__ __forceinline__ void settle64(const KP<P>& p, const Inst<double>& ip, WarpCounts& wc,
+                                         Acc& acc, int inst, unsigned long long pid,
+                                         const PV<P>& xo, double to, const PV<P>& k, double w,
+                                         int l, const TanOf<P>& tau, Cand cand) {
+  PV<P> x = pos_at(p, xo, to, k, p.dt);
+  if (p.L > l + 1) acc.psteps += (unsigned)(p.L - l - 1);
+  for (int c = l + 1; c < p.L; ++c) {
+    if (Draw<P>::first_n(p, pid, c) < ip.n_hi) {
+      if (FEntry<P>* const at = cand()) {
+        FEntry<P> e;
+        static_cast<TanOf<P>&>(e) = tau;
+        e.pid = pid;
+        e.x = x;
+        e.k = k;
+        e.w = w;
+        e.l = ent_pack(c, inst);
+        *at = e;
+      }
+    }
+#pragma unroll
+    for (int d = 0; d < P::D; ++d) x.c[d] = P::stream(x.c[d], k.c[d], p.dtv);
+  }
+  emit_child_final<P, DST>(p, wc, acc, inst, pid, x, k, w, tau);
+}
+
+constexpr unsigned kEFill = 64;      // candidates a warp gathers before it turns to them
+template <class P, int SRC, int DST>
+__device__ __forceinline__ void period_fp64(const KP<P>& p, WarpCounts& wc, Acc& acc, char* work,
+                                            unsigned& first_pairs, unsigned& psteps_first) {
+  using T = typename P::T;
+  const int lane = threadIdx.x & 31;
+  const unsigned g = global_warp();
+  const bool own = g < (unsigned)p.nseg;
+  FEntry<P>* const top = (FEntry<P>*)work;
+  Birth<P>* const buf = (Birth<P>*)(top + kEStack);
+  const CandStack<P> cq{top, p.eq + (size_t)g * p.eseg, own ? kEStack + p.eseg : kEStack};
+  DEntry<P>* const dl = (DEntry<P>*)(p.dq[1] + (size_t)g * p.dseg);
+  const unsigned dcap =
+      own ? (unsigned)((size_t)p.dseg * sizeof(SEntry<P>) / sizeof(DEntry<P>)) : 0u;
+  auto later = [&](const DEntry<P>& s) {
+    const unsigned q = atomicAdd(&wc.d, 1u);
+    if (q < dcap) dl[q] = s;
+    else set_err(p.cnt, ERR_CAP_EQUEUE);
+  };
+  auto cand = [&]() -> FEntry<P>* {
+    const unsigned q = atomicAdd(&wc.e, 1u);
+    if (q < cq.cap) return q < kEStack ? cq.top + q : cq.seg + (q - kEStack);
+    set_err(p.cnt, ERR_CAP_EQUEUE);
+    return nullptr;
+  };
+  unsigned nb = 0;  // accepted events waiting (the same in every lane)
+  SourceInfo<SRC> src;
+  src.load(p);
+  unsigned long long next = g * 32ull;
+  __syncwarp();
+  for (;;) {
+    const unsigned ne = min(wc.e, cq.cap), nd = min(wc.d, dcap);
+    const bool fresh = next < src.n;
+    const unsigned lim = fresh ? 32u : 1u;
+    if (nb >= 32u || (nb && !nd && !ne && lim == 1u)) {
+      // the pairs of accepted events, one per lane
+      const unsigned take = min(nb, 32u);
+      __syncwarp();
+      if ((unsigned)lane < take) {
+        const Birth<P> bb = buf[nb - take + lane];
+        const int l = ent_l(bb.l), inst = ent_inst(bb.l);
+        const Inst<T> ip = inst_of(p, inst);
+        pair_of<P>(p, ip, acc, bb, [&](unsigned long long pid, const PV<P>& k, T w,
+                                   const TanOf<P>& tau) {
+          DEntry<P> ch;
+          ch.n = Draw<P>::first_n(p, pid, l);
+          if (ch.n < ip.n_hi) {
+            static_cast<TanOf<P>&>(ch) = tau;
+            ch.pid = pid;
+            ch.xo = bb.xe;
+            ch.to = ch.t = bb.t;
+            ch.k = k;
+            ch.w = w;
+            ch.l = bb.l;
+            ch.j = 0;
+            later(ch);
+          } else {
+            settle64<P, DST>(p, ip, wc, acc, inst, pid, bb.xe, bb.t, k, w, l, tau, cand);
+          }
+        });
+      }
+      nb -= take;
+    } else if (nd >= 32u || ne >= lim || nd >= lim) {
+      // one event per lane: deferred segments, or first events of candidates
+      const bool def = nd >= 32u || ne < lim;
+      bool made = false;
+      Birth<P> bb;
+      if (def) {
+        const unsigned take = min(nd, 32u), base = nd - take;
+        DEntry<P> s;
+        if ((unsigned)lane < take) s = dl[base + lane];
+        __syncwarp();
+        if (lane == 0) wc.d = base;
+        __syncwarp();
+        if ((unsigned)lane < take) {
+          const unsigned j = s.j & ~kRootFlag;
+          const bool root = (s.j & kRootFlag) != 0u;
+          const int l = ent_l(s.l), inst = ent_inst(s.l);
+          const Inst<T> ip = inst_of(p, inst);
+          const typename Draw<P>::State none{};
+          bool more = false;
+          s.t = P::add(s.t, Draw<P>::life(ip, s.n));
+          if (s.t < p.dt) {
+            made = event_decide<P>(p, ip, inst, s.pid, s.xo, s.to, s.k, s.w, none, l, j, root,
+                                   s.t, s, bb, s.n);
+            more = s.n < ip.n_hi;
+          }
+          if (more) {
+            s.j = (j + 1) | (s.j & kRootFlag);
+            later(s);
+          } else if (!root) {
+            settle64<P, DST>(p, ip, wc, acc, inst, s.pid, s.xo, s.to, s.k, s.w, l, s, cand);
+          }
+        }
+      } else {
+        const unsigned take = min(ne, 32u), base = ne - take;
+        FEntry<P> e;
+        if ((unsigned)lane < take) e = cq.get(base + lane);
+        __syncwarp();
+        if (lane == 0) wc.e = base;
+        __syncwarp();
+        if ((unsigned)lane < take) {
+          const int l = ent_l(e.l), inst = ent_inst(e.l);
+          const Inst<T> ip = inst_of(p, inst);
+          DEntry<P> s;
+          static_cast<TanOf<P>&>(s) = static_cast<const TanOf<P>&>(e);
+          s.pid = e.pid;
+          s.xo = e.x;
+          s.to = (T)0;
+          s.k = e.k;
+          s.w = e.w;
+          s.l = e.l;
+          typename Draw<P>::State st;
+          s.t = Draw<P>::first(p, ip, e.pid, l, (T)0, true, st);
+          if (s.t < p.dt) {
+            ++acc.cand;
+            made = event_decide<P>(p, ip, inst, s.pid, s.xo, s.to, s.k, s.w, st, l, 0u, true,
+                                   s.t, s, bb, s.n);
+            if (s.n < ip.n_hi) {
+              s.j = 1u | kRootFlag;
+              later(s);
+            }
+            first_pairs += made;
+          }
+        }
+      }
+      const unsigned bal = __ballot_sync(kFull, made);
+      if (made) buf[nb + __popc(bal & ((1u << lane) - 1u))] = bb;
+      nb += __popc(bal);
+    } else if (fresh) {
+      unsigned ecount = ne;
+      const unsigned before = acc.psteps;
+      flight_body<P, SRC, DST>(p, wc, acc, src, ecount, cq, next, kEFill);
+      psteps_first += acc.psteps - before;
+      __syncwarp();
+      if (lane == 0) wc.e = ecount;
+    } else {
+      break;
+    }
+    __syncwarp();
+  }
+}
+
+template <class P, int SRC, int DST>
+__global__ void __launch_bounds__(kBlock, kPeriodBlocks) k_period(const KP<P> p_) {
+  const KP<P> p = with_period(p_);
+  extern __shared__ __align__(16) char s_work[];
+  __shared__ unsigned long long red[kWarps];
+  __shared__ WarpCounts s_wc[kWarps];
+  WarpCounts& wc = s_wc[threadIdx.x >> 5];
+  if ((threadIdx.x & 31) == 0) wc.f = wc.e = wc.d = wc.r = wc.flip = 0u;
+  __syncwarp();
+  Acc acc;
+  acc.zero();
+  char* const work = s_work + (threadIdx.x >> 5) * period_warp_bytes<P>();
+  unsigned first_pairs = 0, psteps_first = 0;
+  if constexpr (P::is64) period_fp64<P, SRC, DST>(p, wc, acc, work, first_pairs, psteps_first);
+  else period_fp32<P, SRC, DST>(p, wc, acc, first_pairs, psteps_first);
   block_reduce_add(red, psteps_first, &p.cnt->ledger[LG_PSTEPS0]);
   block_reduce_add(red, acc.cand, &p.cnt->ledger[LG_CAND]);
   block_reduce_add(red, first_pairs, &p.cnt->ledger[LG_PAIRS0]);
   acc.psteps -= psteps_first;  // the offspring's flights
-  reduce_event_tallies(red, acc, p.cnt, DST == DST_BIN2);
+  reduce_event_tallies(red, acc, p.cnt, false);
 }
 
 template <class P, int DST>
@@ -2351,6 +2687,7 @@ KP<P> make_kp(const Ctx* c) {
   p.ecnt = c->ecnt[0];
   p.eq_in = (const FEntry<P>*)c->eq[1];
   p.ecnt_in = c->ecnt[1];
+  p.eq_alt = (FEntry<P>*)c->eq[1];
   p.eseg = (unsigned)c->eseg;
   p.dq[0] = (SEntry<P>*)c->dq[0];
   p.dq[1] = (SEntry<P>*)c->dq[1];
@@ -2456,36 +2793,69 @@ cudaError_t events_any(Ctx* c, const KP<P>& p, int dst, int r) {
   return cudaErrorNotSupported;
 }
 
-// One regenerating period of a lean model in one launch (k_period): the
-// candidate and deferred counts start at zero, the first wave's candidates go
-// to buffer 0 and the rounds alternate between the two buffers.
-template <class P, int DST>
-cudaError_t period(Ctx* c, KP<P> p, size_t cnt_bytes) {
-  static const int occ = occupancy(k_period<P, DST>);
-  cudaError_t e;
-  if ((e = launch_zero(c, c->ecnt[0], cnt_bytes)) != cudaSuccess) return e;
-  if ((e = launch_zero(c, c->dcnt, (size_t)(c->passes + 2) * cnt_bytes)) != cudaSuccess) return e;
-  p.eq = (FEntry<P>*)c->eq[0];
-  p.ecnt = c->ecnt[0];
-  p.eq_alt = (FEntry<P>*)c->eq[1];
+// One chunk in one launch (k_period) of the model F.
+template <class F, int SRC, int DST>
+cudaError_t period(Ctx* c, int l0, int L) {
+  constexpr size_t smem = kWarps * period_warp_bytes<F>();
+  struct Shape {  // once per process: more shared memory than a block may have by default
+    cudaError_t err;
+    int occ = 1;
+    Shape() {
+      err = cudaFuncSetAttribute(k_period<F, SRC, DST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)smem);
+      if (err != cudaSuccess) return;
+      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_period<F, SRC, DST>, kBlock,
+                                                        smem) != cudaSuccess || occ < 1)
+        occ = 1;
+    }
+  };
+  static const Shape shape;
+  if (shape.err != cudaSuccess) return shape.err;
+  KP<F> p = make_kp<F>(c);
+  p.l0 = l0;
+  p.L = L;
+  p.len = L - l0;
   prof_begin(c);
-  k_period<P, DST><<<grid_of(c, occ), kBlock, 0, c->stream>>>(p);
+  k_period<F, SRC, DST><<<grid_of(c, shape.occ), kBlock, smem, c->stream>>>(p);
   prof_end(c);
   c->launches++;
   return cudaGetLastError();
 }
 
-template <class P>
-cudaError_t period_any(Ctx* c, const KP<P>& p, int dst, size_t cnt_bytes) {
-  if constexpr (fused_period<P>()) {
-    if (dst == DST_BIN1) return period<P, DST_BIN1>(c, p, cnt_bytes);
-    // wp's weight sums too (on the 1e8-particle workload 3.97 against 4.72 ms
-    // per period); sp2's record sink runs launch per round
-    if constexpr (P::D == 1 && !P::TG) {
-      if (dst == DST_WSUM) return period<P, DST_WSUM>(c, p, cnt_bytes);
-    }
+template <class F, int SRC>
+cudaError_t period_dst(Ctx* c, int l0, int L, int dst) {
+  if (dst == DST_ARRAY) {
+    if constexpr (SRC == SRC_ARRAY) return period<F, SRC, DST_ARRAY>(c, l0, L);
+    else return cudaErrorNotSupported;
+  }
+  if (dst == DST_BIN1) return period<F, SRC, DST_BIN1>(c, l0, L);
+  // wp's weight sums too (on the 1e8-particle workload 3.97 against 4.72 ms
+  // per period); sp2's record sink runs launch per round
+  if constexpr (F::D == 1 && !F::TG) {
+    if (dst == DST_WSUM) return period<F, SRC, DST_WSUM>(c, l0, L);
   }
   return cudaErrorNotSupported;
+}
+
+// Whether a chunk of this context runs as one launch.  The general FP32 and
+// FP64 models: no event log, the potential of their fused model, and at most
+// one event in two candidate-free intervals (p_any <= 1/2), so that a warp's
+// deferred segments, which it keeps until it has 32, cannot outgrow their
+// segment however the offspring of one interval branch.
+template <class P>
+bool one_launch(const Ctx* c, int src, int dst) {
+  using F = typename FusedModel<P>::type;
+  if constexpr (std::is_void_v<F>) {
+    return false;
+  } else {
+    if (!c->one_launch || dst == DST_BIN2) return false;
+    if (src == SRC_REGEN ? dst == DST_ARRAY : src != SRC_ARRAY) return false;
+    if constexpr (!std::is_same_v<F, P>) {
+      if (c->has_log || !(c->p_max <= 0.5)) return false;
+      if (F::STATIC != (c->ncomp == 0)) return false;
+    }
+    return true;
+  }
 }
 
 // The kernel tables of the 4D model, one thread per row of either type.
@@ -2577,7 +2947,9 @@ struct DriverImpl {
       v.gH = q.H != 0.0 ? 1.0 / q.H : 0.0;
       v.gw0 = 1.0 / q.w;
       v.gw1 = 4.0 * q.w;
-      v.p_hi = q.p_any * (1.0 + 1e-9) + 1e-300;
+      // u0 = n 2^-53 < p_hi exactly when the integer n < ceil(p_hi 2^53)
+      const double p_hi = q.p_any * (1.0 + 1e-9) + 1e-300;
+      v.n_hi = p_hi >= 1.0 ? 1ull << 53 : (unsigned long long)ceil(std::ldexp(p_hi, 53));
       v.p_any_f = (float)q.p_any;
       v.ilq = (float)(1.0 / log1p(-q.p_any));  // -inf for p_any = 0, -0 for p_any = 1
       v.ig0 = q.gamma0 > 0.0 ? (float)(1.0 / q.gamma0) : 0.0f;
@@ -2623,9 +2995,11 @@ struct DriverImpl {
     p.len = L - l0;
     const int rounds = L > l0 ? L - l0 : 1;
     const size_t cnt_bytes = (size_t)c->nseg * sizeof(unsigned);
-    if constexpr (fused_period<P>()) {
-      if (c->one_launch && src == SRC_REGEN && L > l0 && (dst == DST_BIN1 || dst == DST_WSUM))
-        return period_any<P>(c, p, dst, cnt_bytes);
+    if constexpr (!std::is_void_v<typename FusedModel<P>::type>) {
+      using F = typename FusedModel<P>::type;
+      if (L > l0 && one_launch<P>(c, src, dst))
+        return src == SRC_REGEN ? period_dst<F, SRC_REGEN>(c, l0, L, dst)
+                                : period_dst<F, SRC_ARRAY>(c, l0, L, dst);
     }
     for (int r = 0; r < rounds; ++r) {
       p.fq_in = (FEntry<P>*)c->fq[r & 1];

@@ -201,6 +201,8 @@ struct Ctx {
   double* inst_grad;              // read-out (dT/dH, dT/dw) per instance (device)
   // time-dependent potential (wbrw_init_td): components on the device
   int ncomp;
+  int has_log;        // created with an event log (the general kernels)
+  double p_max;       // the largest instance's P(candidate) per interval
   int lean;           // FP32 2D, static potential, no event log (tangents or not)
   void* comp_tab;
   // scratch carve-up
