@@ -950,17 +950,27 @@ wbrw_status wbrw_instance_density(wbrw_ctx* c, int inst, double* density_host,
   if (!c) return WBRW_ERR_ARG;
   if (c->failed) return WBRW_ERR_STATE;
   if (inst < 0 || inst >= c->ninst) return seterr(c, WBRW_ERR_ARG, "no instance %d", inst);
-  wbrw_status st;
+  // the live count of a single run, or of an instance's materialised
+  // particles, counted into scratch; an instance's slots are read apart
+  const unsigned long long* live_dev = nullptr;
+  if (c->ninst == 1) {
+    live_dev = c->state == ST_HISTOGRAM ? &c->cnt->regen_total : &c->cnt->n;
+  } else if (c->state != ST_HISTOGRAM) {
+    unsigned long long* d = (unsigned long long*)(c->obs_scalar + 4);
+    WBRW_TRY(c, launch_zero(c, d, 8), "zero");
+    WBRW_TRY(c, launch_live_instance(c, inst, d), "count");
+    live_dev = d;
+  }
   if (c->state == ST_HISTOGRAM) {
-    WBRW_TRY(c, launch_observables(c, inst, c->buf.grid, nullptr), "observables");
+    WBRW_TRY(c, launch_observables(c, inst, c->buf.grid, nullptr, live_dev), "observables");
   } else if (c->cfg.strategy == WBRW_SP1_PAIR) {
     WBRW_TRY(c, launch_zero(c, c->tmp_grid, (size_t)c->nh * 4), "zero");
     WBRW_TRY(c, drv(c)->bin(c, DST_BIN1, c->tmp_grid, 0), "bin");
-    WBRW_TRY(c, launch_observables(c, inst, c->tmp_grid, nullptr), "observables");
+    WBRW_TRY(c, launch_observables(c, inst, c->tmp_grid, nullptr, live_dev), "observables");
   } else {
     WBRW_TRY(c, launch_zero(c, c->tmp_wsum, (size_t)c->nh * 8), "zero");
     WBRW_TRY(c, drv(c)->bin(c, DST_WSUM, c->tmp_grid, 0), "bin");
-    WBRW_TRY(c, launch_observables(c, inst, nullptr, c->tmp_wsum), "observables");
+    WBRW_TRY(c, launch_observables(c, inst, nullptr, c->tmp_wsum, live_dev), "observables");
   }
   if (density_host)
     WBRW_TRY(c, cudaMemcpyAsync(density_host, c->obs_density,
@@ -969,27 +979,23 @@ wbrw_status wbrw_instance_density(wbrw_ctx* c, int inst, double* density_host,
   if (marginal_x_host)
     WBRW_TRY(c, cudaMemcpyAsync(marginal_x_host, c->obs_marg, (size_t)c->cfg.nx * 8,
                                 cudaMemcpyDeviceToHost, c->stream), "copy marginal");
-  double T = 0;
-  unsigned long long live = 0;
-  WBRW_TRY(c, cudaMemcpyAsync(&T, c->obs_scalar, 8, cudaMemcpyDeviceToHost, c->stream), "copy");
-  if (c->ninst == 1) {
-    WBRW_TRY(c, cudaMemcpyAsync(&live, c->state == ST_HISTOGRAM ? &c->cnt->regen_total
-                                                                : &c->cnt->n,
-                                8, cudaMemcpyDeviceToHost, c->stream), "copy");
-  } else if (c->state == ST_HISTOGRAM) {
-    unsigned long long se[2];
+  // transmission, live count and error word in one copy (each copy into
+  // pageable memory is a round trip of its own)
+  struct {
+    double T;
+    unsigned long long live;
+    long long err;
+  } r = {0.0, 0ull, 0ll};
+  unsigned long long se[2] = {0, 0};
+  WBRW_TRY(c, cudaMemcpyAsync(&r, c->obs_scalar, sizeof(r), cudaMemcpyDeviceToHost, c->stream),
+           "copy");
+  if (c->ninst > 1 && c->state == ST_HISTOGRAM)
     WBRW_TRY(c, cudaMemcpyAsync(se, c->inst_slot + inst, 16, cudaMemcpyDeviceToHost, c->stream),
              "copy");
-    WBRW_TRY(c, cudaStreamSynchronize(c->stream), "synchronise");
-    live = se[1] - se[0];
-  } else {
-    unsigned long long* d = (unsigned long long*)(c->obs_scalar + 1);
-    WBRW_TRY(c, launch_zero(c, d, 8), "zero");
-    WBRW_TRY(c, launch_live_instance(c, inst, d), "count");
-    WBRW_TRY(c, cudaMemcpyAsync(&live, d, 8, cudaMemcpyDeviceToHost, c->stream), "copy");
-  }
-  st = device_status(c);
-  if (st != WBRW_OK) return st;
+  WBRW_TRY(c, cudaStreamSynchronize(c->stream), "synchronise");
+  if (r.err) return device_status(c);
+  const double T = r.T;
+  const unsigned long long live = r.live + (se[1] - se[0]);
   if (transmission) *transmission = T;
   if (live_particles) *live_particles = (long long)live;
   return WBRW_OK;

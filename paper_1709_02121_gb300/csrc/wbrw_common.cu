@@ -1312,71 +1312,153 @@ __global__ void __launch_bounds__(kBlock) k_wp_round(const Counters* c, long lon
 }
 
 // ---------------------------------------------------------------------------
-// Observables: one warp per x-column.
+// Observables.
 // ---------------------------------------------------------------------------
-// counts (int) or wsum (int64, each value times scale) per cell, x-major.
+// The transmission numerator: the columns with centre x > 0 (one block).
+__device__ unsigned long long sum_right(const long long* col, int nx, double xmin, double dx,
+                                        unsigned long long* red) {
+  long long s = 0;
+  for (int ix = threadIdx.x; ix < nx; ix += kBlock) {
+    const double centre = __dadd_rn(xmin, __dmul_rn(__dadd_rn((double)ix, 0.5), dx));
+    if (centre > 0.0) s += __ldcg(col + ix);
+  }
+  unsigned long long t;
+  block_exscan((unsigned long long)s, red, t);
+  return t;
+}
+
+// What a read-out returns, in one piece.
+struct ReadOut {
+  double T;
+  unsigned long long live;
+  long long err;
+};
+
+// counts (int) or wsum (int64, each value times scale) per cell, x-major:
+// density, x-marginal and column sums.  A column is shared by `wpc` warps
+// (1, 2, 4 or 8), so that a few hundred columns fill the chip: one warp each
+// left 1200 x 512 cells to 1200 warps and took 54 us, most of it FP64
+// divisions (1/64 of the FP32 rate); those of 32 empty cells are left out
+// (0 / x = 0).  With `c` the last block also takes the transmission and the
+// rest of the read-out (src_live: the particle count to report).
 __global__ void __launch_bounds__(kBlock) k_obs_cols(const int* counts, const long long* wsum,
                                                      int nx, int nk, double na, double dx,
-                                                     double dk, double scale, double* density,
-                                                     double* marg, long long* col) {
-  const int lane = threadIdx.x & 31;
-  const long long warp = ((long long)blockIdx.x * kBlock + threadIdx.x) >> 5;
-  const long long nwarps = ((long long)gridDim.x * kBlock) >> 5;
-  for (long long ix = warp; ix < nx; ix += nwarps) {
+                                                     double dk, double scale, int wpc,
+                                                     double* density, double* marg,
+                                                     long long* col, Counters* c, double xmin,
+                                                     const unsigned long long* src_live,
+                                                     ReadOut* out) {
+  __shared__ unsigned long long red[kBlock / 32 + 1];
+  __shared__ long long part[kBlock / 32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int cpb = (kBlock / 32) / wpc;  // columns a block takes at a time
+  const double cell = __dmul_rn(__dmul_rn(na, dx), dk);
+  for (int ix0 = blockIdx.x * cpb; ix0 < nx; ix0 += gridDim.x * cpb) {
+    const int ix = ix0 + wid / wpc;
     long long s = 0;
-    for (int ik = lane; ik < nk; ik += 32) {
-      const long long nu = ix * nk + ik;
-      const long long v = wsum ? wsum[nu] : (long long)counts[nu];
-      s += v;
-      if (density)
-        density[nu] = __ddiv_rn(__dmul_rn((double)v, scale), __dmul_rn(__dmul_rn(na, dx), dk));
+    if (ix < nx) {
+      for (int k0 = (wid & (wpc - 1)) * 32; k0 < nk; k0 += wpc * 32) {
+        const int ik = k0 + lane;
+        const long long nu = (long long)ix * nk + ik;
+        const long long v = ik < nk ? (wsum ? wsum[nu] : (long long)counts[nu]) : 0;
+        s += v;
+        if (density) {
+          const bool any = __any_sync(0xFFFFFFFFu, v != 0);
+          const double d = any ? __ddiv_rn(__dmul_rn((double)v, scale), cell) : 0.0;
+          if (ik < nk) density[nu] = d;
+        }
+      }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xFFFFFFFFu, s, o);
-    if (lane == 0) {
-      col[ix] = s;
-      marg[ix] = __ddiv_rn(__dmul_rn((double)s, scale), __dmul_rn(na, dx));
+    __syncthreads();
+    if (lane == 0) part[wid] = s;
+    __syncthreads();
+    if (threadIdx.x < cpb && ix0 + (int)threadIdx.x < nx) {
+      long long t = 0;
+      for (int i = 0; i < wpc; ++i) t += part[threadIdx.x * wpc + i];
+      col[ix0 + threadIdx.x] = t;
+      marg[ix0 + threadIdx.x] = __ddiv_rn(__dmul_rn((double)t, scale), __dmul_rn(na, dx));
     }
   }
+  if (!c || !last_block(&c->scan_ticket)) return;
+  const unsigned long long t = sum_right(col, nx, xmin, dx, red);
+  if (threadIdx.x == 0) {
+    out->T = __ddiv_rn(__dmul_rn((double)(long long)t, scale), na);
+    out->live = src_live ? *src_live : 0ull;
+    out->err = c->err;
+  }
 }
+
+// Warps per column of k_obs_cols.
+int obs_wpc(int nk) { return nk >= 256 ? 8 : nk >= 128 ? 4 : nk >= 64 ? 2 : 1; }
 
 __global__ void __launch_bounds__(kBlock) k_obs_total(const long long* col, int nx, double xmin,
                                                       double dx, double na, double scale,
                                                       double* out) {
   __shared__ unsigned long long red[kBlock / 32 + 1];
-  long long s = 0;
-  for (int ix = threadIdx.x; ix < nx; ix += kBlock) {
-    const double centre = __dadd_rn(xmin, __dmul_rn(__dadd_rn((double)ix, 0.5), dx));
-    if (centre > 0.0) s += col[ix];
-  }
-  unsigned long long t;
-  block_exscan((unsigned long long)s, red, t);
+  const unsigned long long t = sum_right(col, nx, xmin, dx, red);
   if (threadIdx.x == 0)
     out[0] = __ddiv_rn(__dmul_rn((double)(long long)t, scale), na);
 }
 
-// Transmission of each instance (one block each): the sum of its counts
-// over the cells with centre x > 0, divided by its N_alpha.  The cells with
-// centre x > 0 are the columns ix >= ix0, a contiguous range.
-__global__ void __launch_bounds__(kBlock) k_obs_trans(const int* counts, int nx, int nk,
-                                                      double xmin, double dx, const double* na,
-                                                      double* out) {
-  __shared__ unsigned long long red[kBlock / 32 + 1];
+// The first column with centre x > 0, i.e. the columns ix >= ix0 (a
+// contiguous range).
+__device__ int first_right(int nx, double xmin, double dx) {
   __shared__ int s_ix0;
   if (threadIdx.x == 0) {
-    int ix0 = nx;
-    for (int ix = 0; ix < nx; ++ix)
-      if (__dadd_rn(xmin, __dmul_rn(__dadd_rn((double)ix, 0.5), dx)) > 0.0) { ix0 = ix; break; }
-    s_ix0 = ix0;
+    int lo = 0, hi = nx;  // the centres increase
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (__dadd_rn(xmin, __dmul_rn(__dadd_rn((double)mid, 0.5), dx)) > 0.0) hi = mid;
+      else lo = mid + 1;
+    }
+    s_ix0 = lo;
   }
   __syncthreads();
-  const long long nhi = (long long)nx * nk;
-  const int* g = counts + (long long)blockIdx.x * nhi;
+  return s_ix0;
+}
+
+// Sums of one instance's cells right of x = 0, cut into gridDim.x pieces per
+// instance (blockIdx.y), four loads a thread in flight, added to acc (zeroed
+// by the caller).  One block per instance read 256 instances' 79 MB at 1.1 TB/s.
+template <class T>
+__device__ void sum_cells_right(const T* g, int nx, int nk, int ix0, unsigned long long* red,
+                                unsigned long long* acc) {
+  const long long a = (long long)ix0 * nk, n = (long long)nx * nk - a;
+  const long long per = (n + gridDim.x - 1) / gridDim.x;
+  const long long b0 = a + (long long)blockIdx.x * per;
+  const long long b1 = b0 + per < a + n ? b0 + per : a + n;
   long long s = 0;
-  for (long long nu = (long long)s_ix0 * nk + threadIdx.x; nu < nhi; nu += kBlock) s += g[nu];
+  for (long long nu = b0 + threadIdx.x; nu < b1; nu += 4 * kBlock) {
+    T v[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = nu + i * kBlock < b1 ? g[nu + i * kBlock] : (T)0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) s += (long long)v[i];
+  }
   unsigned long long t;
   block_exscan((unsigned long long)s, red, t);
-  if (threadIdx.x == 0) out[blockIdx.x] = __ddiv_rn((double)(long long)t, na[blockIdx.x]);
+  if (threadIdx.x == 0 && t) atomicAdd(acc, t);
+}
+
+// Transmission of each instance: the sum of its counts over the cells with
+// centre x > 0, divided by its N_alpha.
+__global__ void __launch_bounds__(kBlock) k_obs_trans(const int* counts, int nx, int nk,
+                                                      double xmin, double dx,
+                                                      unsigned long long* acc) {
+  __shared__ unsigned long long red[kBlock / 32 + 1];
+  const int ix0 = first_right(nx, xmin, dx);
+  sum_cells_right(counts + (long long)blockIdx.y * nx * nk, nx, nk, ix0, red, acc + blockIdx.y);
+}
+
+// The sums (integers in units of `unit`) over N_alpha, in place.
+__global__ void __launch_bounds__(kBlock) k_obs_over_na(unsigned long long* acc, int n, int per,
+                                                        double unit, const double* na) {
+  const int i = blockIdx.x * kBlock + threadIdx.x;
+  if (i >= n) return;
+  const double v = __dmul_rn((double)(long long)acc[i], unit);
+  ((double*)acc)[i] = __ddiv_rn(v, na[i / per]);
 }
 
 // Particles of one instance in the arrays: its base slots plus the offspring
@@ -1398,52 +1480,45 @@ __global__ void __launch_bounds__(kBlock) k_live_inst(const Counters* c,
 }
 
 // The 4D counts summed over electron 2: red[ix1 nk + ik1] =
-// sum over (ix2, ik2) of counts[((ix1 nx + ix2) nk + ik1) nk + ik2], one warp
-// per output.
+// sum over (ix2, ik2) of counts[((ix1 nx + ix2) nk + ik1) nk + ik2].  A warp
+// sums one row (ix1, ix2, ik1) of nk cells at a time and adds it to its
+// output (zeroed by the caller) when it has taken kRed4 of them, the rows of
+// one output eight loads ahead: one warp per output left 64 x 64 outputs to
+// 4096 warps of 128 dependent loads each (33 us of 67 MB).
+constexpr int kRed4 = 8;
 __global__ void __launch_bounds__(kBlock) k_reduce4(const int* counts, int nx, int nk,
                                                     long long* red) {
   const int lane = threadIdx.x & 31;
   const long long warp = ((long long)blockIdx.x * kBlock + threadIdx.x) >> 5;
   const long long nwarps = ((long long)gridDim.x * kBlock) >> 5;
-  for (long long o = warp; o < (long long)nx * nk; o += nwarps) {
-    const long long ix1 = o / nk, ik1 = o % nk;
+  const int parts = (nx + kRed4 - 1) / kRed4;
+  for (long long w = warp; w < (long long)nx * parts * nk; w += nwarps) {
+    const long long ik1 = w % nk, q = w / nk;
+    const long long ix1 = q / parts;
+    const int x0 = (int)(q % parts) * kRed4;
     long long s = 0;
-    for (long long ix2 = 0; ix2 < nx; ++ix2) {
-      const int* row = counts + ((ix1 * nx + ix2) * nk + ik1) * nk;
-      for (int ik2 = lane; ik2 < nk; ik2 += 32) s += row[ik2];
-    }
+    for (int ik2 = lane; ik2 < nk; ik2 += 32) {
+      int v[kRed4];
 #pragma unroll
-    for (int d = 16; d > 0; d >>= 1) s += __shfl_down_sync(0xFFFFFFFFu, s, d);
-    if (lane == 0) red[o] = s;
+      for (int i = 0; i < kRed4; ++i)
+        v[i] = x0 + i < nx ? counts[((ix1 * nx + x0 + i) * nk + ik1) * nk + ik2] : 0;
+#pragma unroll
+      for (int i = 0; i < kRed4; ++i) s += v[i];
+    }
+    s = (long long)warp_sum((unsigned long long)s);
+    if (lane == 0 && s) atomicAdd((unsigned long long*)(red + ix1 * nk + ik1), (unsigned long long)s);
   }
 }
 
-// (dT/dH, dT/dw) of each instance (one block each): the tangent histogram
-// summed over the cells with centre x > 0, times 2^-32, over N_alpha.
+// (dT/dH, dT/dw) of each instance: the tangent histogram (2^-32 units)
+// summed over the cells with centre x > 0.
 __global__ void __launch_bounds__(kBlock) k_obs_tgrad(const long long* dH, const long long* dw,
                                                       int nx, int nk, double xmin, double dx,
-                                                      const double* na, double* out) {
+                                                      unsigned long long* acc) {
   __shared__ unsigned long long red[kBlock / 32 + 1];
-  __shared__ int s_ix0;
-  if (threadIdx.x == 0) {
-    int ix0 = nx;
-    for (int ix = 0; ix < nx; ++ix)
-      if (__dadd_rn(xmin, __dmul_rn(__dadd_rn((double)ix, 0.5), dx)) > 0.0) { ix0 = ix; break; }
-    s_ix0 = ix0;
-  }
-  __syncthreads();
-  const long long nhi = (long long)nx * nk;
-  for (int d = 0; d < 2; ++d) {
-    const long long* g = (d ? dw : dH) + (long long)blockIdx.x * nhi;
-    long long acc = 0;
-    for (long long nu = (long long)s_ix0 * nk + threadIdx.x; nu < nhi; nu += kBlock) acc += g[nu];
-    unsigned long long t;
-    block_exscan((unsigned long long)acc, red, t);
-    if (threadIdx.x == 0)
-      out[2 * blockIdx.x + d] =
-          __ddiv_rn(__dmul_rn((double)(long long)t, 1.0 / 4294967296.0), na[blockIdx.x]);
-    __syncthreads();
-  }
+  const int ix0 = first_right(nx, xmin, dx);
+  const long long off = (long long)(blockIdx.y >> 1) * nx * nk;
+  sum_cells_right(((blockIdx.y & 1) ? dw : dH) + off, nx, nk, ix0, red, acc + blockIdx.y);
 }
 
 int grid_cap(Ctx* c, int per_sm) { return c->num_sms * per_sm; }
@@ -1594,7 +1669,8 @@ cudaError_t launch_wp_round(Ctx* c, int epoch_delta) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_observables(Ctx* c, int inst, const int* counts, const long long* wsum) {
+cudaError_t launch_observables(Ctx* c, int inst, const int* counts, const long long* wsum,
+                               const unsigned long long* live) {
   const double na = (double)c->ih[inst].n_alpha;
   const int g = grid_cap(c, 4);
   const long long off = (long long)inst * c->nhi;
@@ -1602,24 +1678,38 @@ cudaError_t launch_observables(Ctx* c, int inst, const int* counts, const long l
   const long long* ws = wsum ? wsum + off : nullptr;
   double scale = wsum ? 1.0 / 2147483648.0 : 1.0;
   if (c->dim == 4 && cn) {  // electron 1's reduced counts
-    k_reduce4<<<g, kBlock, 0, c->stream>>>(cn, c->cfg.nx, c->cfg.nk, c->obs_red);
+    const cudaError_t e = launch_zero(c, c->obs_red, (size_t)c->cfg.nx * c->cfg.nk * 8);
+    if (e != cudaSuccess) return e;
+    k_reduce4<<<2 * g, kBlock, 0, c->stream>>>(cn, c->cfg.nx, c->cfg.nk, c->obs_red);
     c->launches++;
     cn = nullptr;
     ws = c->obs_red;
     scale = 1.0;
   }
-  k_obs_cols<<<g, kBlock, 0, c->stream>>>(cn, ws, c->cfg.nx, c->cfg.nk, na, c->dx, c->dk, scale,
-                                          c->obs_density, c->obs_marg, c->obs_col);
-  k_obs_total<<<1, kBlock, 0, c->stream>>>(c->obs_col, c->cfg.nx, c->cfg.xmin, c->dx, na,
-                                           scale, c->obs_scalar);
-  c->launches += 2;
+  const int wpc = obs_wpc(c->cfg.nk), cpb = kBlock / 32 / wpc;
+  const int blocks = (c->cfg.nx + cpb - 1) / cpb;
+  k_obs_cols<<<blocks < 2 * g ? blocks : 2 * g, kBlock, 0, c->stream>>>(
+      cn, ws, c->cfg.nx, c->cfg.nk, na, c->dx, c->dk, scale, wpc, c->obs_density, c->obs_marg,
+      c->obs_col, c->cnt, c->cfg.xmin, live, (ReadOut*)c->obs_scalar);
+  c->launches += 1;
   return cudaGetLastError();
 }
 
+// Pieces per instance of the sums over cells: about two blocks per SM in
+// all, of at least 1024 cells each.
+static int pieces(const Ctx* c, int rows) {
+  const long long want = (2ll * c->num_sms + rows - 1) / rows, most = (c->nhi + 1023) / 1024;
+  return (int)(want < most ? want : most);
+}
+
 cudaError_t launch_transmissions(Ctx* c, const int* counts, double* out) {
-  k_obs_trans<<<c->ninst, kBlock, 0, c->stream>>>(counts, c->cfg.nx, c->cfg.nk, c->cfg.xmin,
-                                                  c->dx, c->inst_na, out);
-  c->launches++;
+  cudaError_t e = launch_zero(c, out, (size_t)c->ninst * 8);
+  if (e != cudaSuccess) return e;
+  k_obs_trans<<<dim3(pieces(c, c->ninst), c->ninst), kBlock, 0, c->stream>>>(
+      counts, c->cfg.nx, c->cfg.nk, c->cfg.xmin, c->dx, (unsigned long long*)out);
+  k_obs_over_na<<<(c->ninst + kBlock - 1) / kBlock, kBlock, 0, c->stream>>>(
+      (unsigned long long*)out, c->ninst, 1, 1.0, c->inst_na);
+  c->launches += 2;
   return cudaGetLastError();
 }
 
@@ -1632,9 +1722,15 @@ cudaError_t launch_scan_tangent(Ctx* c) {
 }
 
 cudaError_t launch_transmission_gradients(Ctx* c) {
-  k_obs_tgrad<<<c->ninst, kBlock, 0, c->stream>>>(c->dgrid[0], c->dgrid[1], c->cfg.nx, c->cfg.nk,
-                                                  c->cfg.xmin, c->dx, c->inst_na, c->inst_grad);
-  c->launches++;
+  cudaError_t e = launch_zero(c, c->inst_grad, (size_t)c->ninst * 16);
+  if (e != cudaSuccess) return e;
+  const int rows = 2 * c->ninst;
+  k_obs_tgrad<<<dim3(pieces(c, rows), rows), kBlock, 0, c->stream>>>(
+      c->dgrid[0], c->dgrid[1], c->cfg.nx, c->cfg.nk, c->cfg.xmin, c->dx,
+      (unsigned long long*)c->inst_grad);
+  k_obs_over_na<<<(rows + kBlock - 1) / kBlock, kBlock, 0, c->stream>>>(
+      (unsigned long long*)c->inst_grad, rows, 2, 1.0 / 4294967296.0, c->inst_na);
+  c->launches += 2;
   return cudaGetLastError();
 }
 
@@ -1712,8 +1808,11 @@ extern "C" wbrw_status wbrw_observables_static(const int* grid, int nx, int nk, 
   // Each launch is checked on its own.  cudaGetLastError also returns (and
   // clears) an error that an earlier runtime call of the caller left
   // pending; such an error is reported here as WBRW_ERR_CUDA.
-  wbrw::k_obs_cols<<<4 * sms, wbrw::kBlock, 0, s>>>(grid, nullptr, nx, nk, na, dx, dk, 1.0, density,
-                                                    marginal_x, col);
+  const int wpc = wbrw::obs_wpc(nk), cpb = wbrw::kBlock / 32 / wpc;
+  const int blocks = (nx + cpb - 1) / cpb;
+  wbrw::k_obs_cols<<<blocks < 8 * sms ? blocks : 8 * sms, wbrw::kBlock, 0, s>>>(
+      grid, nullptr, nx, nk, na, dx, dk, 1.0, wpc, density, marginal_x, col, nullptr, xmin, nullptr,
+      nullptr);
   if (cudaGetLastError() != cudaSuccess) return WBRW_ERR_CUDA;
   wbrw::k_obs_total<<<1, wbrw::kBlock, 0, s>>>(col, nx, xmin, dx, na, 1.0, transmission);
   if (cudaGetLastError() != cudaSuccess) return WBRW_ERR_CUDA;

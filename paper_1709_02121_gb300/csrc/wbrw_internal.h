@@ -341,8 +341,10 @@ cudaError_t launch_boot(Ctx*, int epoch_delta);
 // wp: Alg. 3's rounding of the weighted histogram tmp_wsum into the grid.
 cudaError_t launch_wp_round(Ctx*, int epoch_delta);
 // Observables of instance `inst` from the counts / Q1.31 weight sums of all
-// instances (one of the two is NULL).
-cudaError_t launch_observables(Ctx*, int inst, const int* counts, const long long* wsum);
+// instances (one of the two is NULL).  c->obs_scalar receives the
+// transmission, *live (device; 0 if NULL) and the error word, 8 bytes each.
+cudaError_t launch_observables(Ctx*, int inst, const int* counts, const long long* wsum,
+                               const unsigned long long* live = nullptr);
 // Transmission of every instance into out (ninst doubles, device).
 cudaError_t launch_transmissions(Ctx*, const int* counts, double* out);
 cudaError_t launch_zero(Ctx*, void* p, size_t bytes);
