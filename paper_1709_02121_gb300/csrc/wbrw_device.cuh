@@ -277,9 +277,11 @@ struct Tab4 {
   const T* xi[2];     // ny per type
   const T* cdf[2];    // ny x nkap per type
   const int* guide[2];  // FP32: ny x (kTabGuide + 1) per type (see k_tab4_guide)
-  double Y[2], inv_dy[2];
-  double gam[2];      // component rates gamma_t (one-body twice, interaction once)
-  double xc;          // nucleus
+  // rounded to T on the host: converted in the kernel, each was an FP64
+  // instruction per event, at 1/64 of the FP32 rate
+  T Y[2], inv_dy[2];
+  T gam[2];           // component rates gamma_t (one-body twice, interaction once)
+  T xc;               // nucleus
   T kap0, dkap;       // -K, dkappa
   int ny, nkap;
 };
@@ -543,17 +545,17 @@ __device__ __forceinline__ bool table_kick(const KP<P>& p, typename P::T Gam, co
                                            typename P::T& kap, typename P::T& prob) {
   using T = typename P::T;
   const Tab4<T>& tb = p.tab;
-  const T g_ne = (T)tb.gam[0], g_ee = (T)tb.gam[1];
+  const T g_ne = tb.gam[0], g_ee = tb.gam[1];
   const T v = P::mul(uc, Gam);
   const int m = v < g_ne ? 0 : (v < P::mul((T)2, g_ne) ? 1 : 2);
   comp = m;
   const int t = m == 2 ? 1 : 0;
-  const T xc = (T)tb.xc;
+  const T xc = tb.xc;
   const T y = m == 0 ? P::sub(xe.c[0], xc)
                      : (m == 1 ? P::sub(xe.c[P::D - 1], xc) : P::sub(xe.c[0], xe.c[P::D - 1]));
   const T g = m == 2 ? g_ee : g_ne;
   // (selects, not indexing by t: the parameters stay out of local memory)
-  const T sp = P::mul(P::add(y, (T)(t ? tb.Y[1] : tb.Y[0])), (T)(t ? tb.inv_dy[1] : tb.inv_dy[0]));
+  const T sp = P::mul(P::add(y, t ? tb.Y[1] : tb.Y[0]), t ? tb.inv_dy[1] : tb.inv_dy[0]);
   int i;
   T th;
   if (!(sp > (T)0)) {
@@ -2651,11 +2653,11 @@ KP<P> make_kp(const Ctx* c) {
     p.tab.xi[t] = (const T*)c->tab_xi[t];
     p.tab.cdf[t] = (const T*)c->tab_cdf[t];
     p.tab.guide[t] = c->tab_guide[t];
-    p.tab.Y[t] = c->tab_Y[t];
-    p.tab.inv_dy[t] = c->tab_inv_dy[t];
-    p.tab.gam[t] = c->tab_gam[t];
+    p.tab.Y[t] = (T)c->tab_Y[t];
+    p.tab.inv_dy[t] = (T)c->tab_inv_dy[t];
+    p.tab.gam[t] = (T)c->tab_gam[t];
   }
-  p.tab.xc = c->pot.xc;
+  p.tab.xc = (T)c->pot.xc;
   p.tab.kap0 = (T)(-c->tab_K);
   p.tab.dkap = (T)c->tab_dkap;
   p.tab.ny = c->tab_ny;
