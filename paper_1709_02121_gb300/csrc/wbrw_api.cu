@@ -726,10 +726,21 @@ wbrw_status create(const wbrw_config* config, const wbrw_potential* pot, int nin
   c->obs_red = (long long*)(base + L.obs_red);
   c->ncomp = ncomp;
   c->comp_tab = base + L.tabs + kTabCompOff;
-  if (ncomp > 0 && cudaMemcpyAsync(c->comp_tab, comps, (size_t)ncomp * sizeof(Comp),
-                                   cudaMemcpyHostToDevice, c->stream) != cudaSuccess) {
-    free_ctx(c);
-    return WBRW_ERR_CUDA;
+  if (ncomp > 0) {
+    // in the run's precision, rounded here: converted in the kernels, each
+    // of an event's eight fields was an FP64 instruction (1/64 of the FP32 rate)
+    CompOf<float> cf[kMaxComp];
+    for (int m = 0; m < ncomp; ++m)
+      cf[m] = {(float)comps[m].a, (float)comps[m].b, (float)comps[m].om, (float)comps[m].ph,
+               (float)comps[m].sig_k, (float)comps[m].xc, (float)comps[m].gam,
+               (float)comps[m].hg};
+    const bool f32 = config->precision == WBRW_FP32;
+    if (cudaMemcpyAsync(c->comp_tab, f32 ? (const void*)cf : (const void*)comps,
+                        (size_t)ncomp * (f32 ? sizeof(cf[0]) : sizeof(Comp)),
+                        cudaMemcpyHostToDevice, c->stream) != cudaSuccess) {
+      free_ctx(c);
+      return WBRW_ERR_CUDA;
+    }
   }
   c->tangent = config->tangent;
   c->inst_grad = (double*)(base + L.tabs + kTabGradOff);

@@ -46,6 +46,7 @@ constexpr size_t kTabGradOff = kTabTSlotOff + (size_t)(kMaxInst + 1) * 8;
 constexpr size_t kTabCompOff = kTabGradOff + (size_t)kMaxInst * 16;
 constexpr int kMaxComp = WBRW_MAX_COMPONENTS;  // components of a time-dependent V
 constexpr size_t kTabBytes = kTabCompOff + (size_t)kMaxComp * 64;
+static_assert(8 * sizeof(double) <= 64, "component records");
 
 // SRC_TREGEN: the tangent mode's sign-0 particles regenerated from the
 // tangent histogram (a second plan).
@@ -148,9 +149,11 @@ constexpr int kMaxGraphs = 4;
 // One Gaussian component of a time-dependent potential, as the kernels read
 // it: V_m(x, t) = (a + b cos(om t + ph)) exp(-(x - xc)^2/(2 w^2)),
 // sig_k = 1/(2w), gam = (|a| + |b|)/hbar (its majorant rate), hg = hbar gam.
-struct Comp {
-  double a, b, om, ph, sig_k, xc, gam, hg;
+template <class T>
+struct CompOf {
+  T a, b, om, ph, sig_k, xc, gam, hg;
 };
+using Comp = CompOf<double>;
 
 // One instance of a batch, host FP64 (Sec. 4.2 / Remark 3 / Sec. 3.2).
 struct InstHost {
