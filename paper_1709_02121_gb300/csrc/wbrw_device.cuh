@@ -1378,6 +1378,26 @@ struct CandStack {
   }
 };
 
+// ... or (FP32 one-launch flights of few particles) the warp's ring: its
+// segments of both candidate buffers, one after the other.  Positions are
+// numbers modulo 2 half; head is the first entry not yet taken.
+template <class P>
+struct CandRing {
+  static constexpr bool STACK = false;
+  FEntry<P>* seg0;
+  FEntry<P>* seg1;
+  unsigned half, head;
+  __device__ __forceinline__ FEntry<P>* at(unsigned q) const {  // q < 4 half
+    if (q >= 2u * half) q -= 2u * half;
+    return q < half ? seg0 + q : seg1 + (q - half);
+  }
+  __device__ __forceinline__ bool put(unsigned q, const FEntry<P>& e) const {
+    if (q - head >= 2u * half) return false;
+    *at(q) = e;
+    return true;
+  }
+};
+
 // Append one candidate entry per flagged lane (interval c, the position
 // streamed from the lane's interval ls to c) to the warp's candidates;
 // ecount is their count, held in a register by every lane.  Every lane of
@@ -2311,6 +2331,219 @@ __device__ __forceinline__ void period_fp32(const KP<P>& p, WarpCounts& wc, Acc&
   }
 }
 
+// FP32, few particles a warp (period_ring).  A round's part-filled passes
+// (candidates, accepted events, deferred segments) cost a warp of a few
+// hundred particles more than its full ones, so here the warp's candidates
+// are one list, taken in order, and 32 of a list are taken whenever one holds
+// 32; part-filled passes are made only when none does.
+template <class P, int DST, class Cand>
+__device__ __forceinline__ void settle_to(const KP<P>& p, WarpCounts& wc, Acc& acc, int inst,
+                                          unsigned long long pid, const PV<P>& xo, float to,
+                                          const PV<P>& k, float w, int l, const TanOf<P>& tau,
+                                          float t_next, Cand cand) {
+  // as settle's FP32 part
+  PV<P> x = pos_at(p, xo, to, k, p.dt);
+  const int n = p.L - l - 1;
+  if (n > 0) {
+    acc.psteps += (unsigned)n;
+    const float q = fmaxf(floorf(t_next * p.inv_dt), 1.0f);
+    const int c = q < (float)(n + 1) ? l + (int)q : p.L;
+    if (c < p.L) {
+      FEntry<P> e;
+      static_cast<TanOf<P>&>(e) = tau;
+      e.pid = pid;
+#pragma unroll
+      for (int d = 0; d < P::D; ++d) e.x.c[d] = stream_n<P>(x.c[d], k.c[d], p.dtv, c - l - 1);
+      e.k = k;
+      e.w = w;
+      e.l = ent_pack(c, inst);
+      cand(e);
+    }
+#pragma unroll
+    for (int d = 0; d < P::D; ++d) x.c[d] = stream_n<P>(x.c[d], k.c[d], p.dtv, n);
+  }
+  emit_child_final<P, DST>(p, wc, acc, inst, pid, x, k, w, tau);
+}
+
+template <class P, class Cand>
+__device__ __forceinline__ void chain_to(const KP<P>& p, const SEntry<P>& s, Cand cand) {
+  // as chain_next
+  const int l = ent_l(s.l);
+  const float q = fmaxf(floorf(s.t * p.inv_dt), 1.0f);  // s.t >= dt
+  if (q < (float)(p.L - l)) {
+    const int c = l + (int)q;
+    FEntry<P> e;
+    static_cast<TanOf<P>&>(e) = static_cast<const TanOf<P>&>(s);
+    e.pid = s.pid;
+#pragma unroll
+    for (int d = 0; d < P::D; ++d) e.x.c[d] = stream_n<P>(s.xo.c[d], s.k.c[d], p.dtv, c - l);
+    e.k = s.k;
+    e.w = s.w;
+    e.l = ent_pack(c, ent_inst(s.l));
+    cand(e);
+  }
+}
+
+template <class P, int SRC, int DST>
+__device__ __forceinline__ void period_ring(const KP<P>& p, WarpCounts& wc, Acc& acc,
+                                            unsigned& first_pairs, unsigned& psteps_first) {
+  using T = typename P::T;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const unsigned g = global_warp();
+  const bool own = g < (unsigned)p.nseg;
+  __shared__ Birth<P> s_birth[kWarps][kBirths];
+  __shared__ __align__(16) FEntry<P> s_stage[kWarps][64];
+  static_assert(sizeof(s_birth) + sizeof(s_stage) + 512 <= 48 * 1024,
+                "a block declares at most 48 KB of static shared memory");
+  Birth<P>* const buf = s_birth[wid];
+  FEntry<P>* const stage = s_stage[wid];
+  CandRing<P> cq{p.eq + (size_t)g * p.eseg, p.eq_alt + (size_t)g * p.eseg, own ? p.eseg : 0u, 0u};
+  SEntry<P>* const dl = p.dq[1] + (size_t)g * p.dseg;
+  const unsigned dcap = own ? p.dseg : 0u;
+  auto later = [&](const SEntry<P>& s) {
+    const unsigned q = atomicAdd(&wc.d, 1u);
+    if (q < dcap) dl[q] = s;
+    else set_err(p.cnt, ERR_CAP_EQUEUE);
+  };
+  auto cand = [&](const FEntry<P>& e) {
+    const unsigned q = atomicAdd(&wc.e, 1u);
+    if (!cq.put(q, e)) set_err(p.cnt, ERR_CAP_EQUEUE);
+  };
+  {
+    unsigned ecount = 0;
+    const unsigned long long nwarps = (unsigned long long)gridDim.x * kWarps;
+    SourceInfo<SRC> src;
+    src.load(p);
+    unsigned long long next = g * 32ull;
+    flight_body<P, SRC, DST>(p, wc, acc, src, ecount, cq, next, nwarps);
+    if constexpr (P::TG && SRC == SRC_REGEN) {  // the tangent particles of the same histogram
+      SourceInfo<SRC_TREGEN> tsrc;
+      tsrc.load(p);
+      next = g * 32ull;
+      flight_body<P, SRC_TREGEN, DST>(p, wc, acc, tsrc, ecount, cq, next, nwarps);
+    }
+    __syncwarp();
+    if (lane == 0) wc.e = min(ecount, 2u * cq.half);
+    __syncwarp();
+  }
+  psteps_first = acc.psteps;
+  unsigned nb = 0;            // accepted events waiting (the same in every lane)
+  unsigned pf = 0, flip = 0;  // candidates from cq.head on staged in half `flip` of stage
+  for (;;) {
+    const unsigned ne = min(wc.e - cq.head, 2u * cq.half), nd = min(wc.d, dcap);
+    if (nb >= 32u || (nb && !nd && !ne)) {
+      // the pairs of accepted events, one per lane
+      const unsigned take = min(nb, 32u);
+      __syncwarp();
+      if ((unsigned)lane < take) {
+        const Birth<P> bb = buf[nb - take + lane];
+        const int l = ent_l(bb.l), inst = ent_inst(bb.l);
+        const Inst<T> ip = inst_of(p, inst);
+        pair_of<P>(p, ip, acc, bb, [&](unsigned long long pid, const PV<P>& k, T w,
+                                       const TanOf<P>& tau) {
+          SEntry<P> ch;
+          static_cast<TanOf<P>&>(ch) = tau;
+          ch.pid = pid;
+          ch.xo = bb.xe;
+          ch.to = bb.t;
+          ch.k = k;
+          ch.w = w;
+          ch.l = bb.l;
+          ch.j = 0;
+          ch.t = Draw<P>::first(p, ip, pid, l, bb.t, false, ch.st);
+          if (ch.t < p.dt) later(ch);
+          else settle_to<P, DST>(p, wc, acc, inst, pid, bb.xe, bb.t, k, w, l, tau, ch.t, cand);
+        });
+      }
+      nb -= take;
+    } else if (ne || nd) {
+      // one event per lane: deferred segments, or first events of candidates
+      bool made = false;
+      Birth<P> bb;
+      if (nd >= 32u || !ne) {
+        const unsigned take = min(nd, 32u), base = nd - take;
+        SEntry<P> s;
+        if ((unsigned)lane < take) s = dl[base + lane];
+        __syncwarp();
+        if (lane == 0) wc.d = base;
+        __syncwarp();
+        if ((unsigned)lane < take) {
+          const unsigned j = s.j & ~kRootFlag;
+          const bool root = (s.j & kRootFlag) != 0u;
+          const int l = ent_l(s.l), inst = ent_inst(s.l);
+          const Inst<T> ip = inst_of(p, inst);
+          T gap;
+          made = event_decide<P>(p, ip, inst, s.pid, s.xo, s.to, s.k, s.w, s.st, l, j, root, s.t,
+                                 s, bb, gap);
+          s.t = P::add(s.t, gap);
+          if (s.t < p.dt) {
+            s.j = (j + 1) | (s.j & kRootFlag);
+            later(s);
+          } else if (!root) {
+            settle_to<P, DST>(p, wc, acc, inst, s.pid, s.xo, s.to, s.k, s.w, l, s, s.t, cand);
+          } else {
+            chain_to<P>(p, s, cand);
+          }
+        }
+      } else {
+        const unsigned take = min(ne, 32u);
+        // staged while the last group was processed, or (written since, or
+        // the first) read here; then the next group's copies start
+        cp_async_wait<0>();
+        FEntry<P> e;
+        if ((unsigned)lane < take)
+          e = (unsigned)lane < pf ? stage[flip * 32u + lane] : *cq.at(cq.head + lane);
+        cq.head += take;
+        if (cq.head >= 2u * cq.half) {
+          // positions and numbers start over together
+          cq.head -= 2u * cq.half;
+          __syncwarp();
+          if (lane == 0) wc.e -= 2u * cq.half;
+          __syncwarp();
+        }
+        flip ^= 1u;
+        pf = min(ne - take, 32u);
+        if ((unsigned)lane < pf)
+          copy_entry_async<P>(&stage[flip * 32u + lane], cq.at(cq.head + lane));
+        cp_async_commit();
+        if ((unsigned)lane < take) {
+          const int l = ent_l(e.l), inst = ent_inst(e.l);
+          const Inst<T> ip = inst_of(p, inst);
+          SEntry<P> s;
+          static_cast<TanOf<P>&>(s) = static_cast<const TanOf<P>&>(e);
+          s.pid = e.pid;
+          s.xo = e.x;
+          s.to = (T)0;
+          s.k = e.k;
+          s.w = e.w;
+          s.l = e.l;
+          s.t = Draw<P>::first(p, ip, e.pid, l, (T)0, true, s.st);
+          if (s.t < p.dt) {
+            ++acc.cand;
+            T gap;
+            made = event_decide<P>(p, ip, inst, s.pid, s.xo, s.to, s.k, s.w, s.st, l, 0u, true,
+                                   s.t, s, bb, gap);
+            s.t = P::add(s.t, gap);
+            if (s.t < p.dt) {
+              s.j = 1u | kRootFlag;
+              later(s);
+            } else {
+              chain_to<P>(p, s, cand);
+            }
+            first_pairs += made;
+          }
+        }
+      }
+      const unsigned bal = __ballot_sync(kFull, made);
+      if (made) buf[nb + __popc(bal & ((1u << lane) - 1u))] = bb;
+      nb += __popc(bal);
+    } else {
+      break;
+    }
+    __syncwarp();
+  }
+}
+
 // FP64 (period_fp64): FP64 instructions run at 1/64 of the FP32 rate here and
 // cost the same however few lanes are at work, so the lanes are kept filled
 // and the logarithms few:
@@ -2496,7 +2729,7 @@ __device__ __forceinline__ void period_fp64(const KP<P>& p, WarpCounts& wc, Acc&
   }
 }
 
-template <class P, int SRC, int DST>
+template <class P, int SRC, int DST, bool RING>
 __global__ void __launch_bounds__(kBlock, kPeriodBlocks) k_period(const KP<P> p_) {
   const KP<P> p = with_period(p_);
   extern __shared__ __align__(16) char s_work[];
@@ -2510,6 +2743,7 @@ __global__ void __launch_bounds__(kBlock, kPeriodBlocks) k_period(const KP<P> p_
   char* const work = s_work + (threadIdx.x >> 5) * period_warp_bytes<P>();
   unsigned first_pairs = 0, psteps_first = 0;
   if constexpr (P::is64) period_fp64<P, SRC, DST>(p, wc, acc, work, first_pairs, psteps_first);
+  else if constexpr (RING) period_ring<P, SRC, DST>(p, wc, acc, first_pairs, psteps_first);
   else period_fp32<P, SRC, DST>(p, wc, acc, first_pairs, psteps_first);
   block_reduce_add(red, psteps_first, &p.cnt->ledger[LG_PSTEPS0]);
   block_reduce_add(red, acc.cand, &p.cnt->ledger[LG_CAND]);
@@ -2857,18 +3091,39 @@ cudaError_t events_any(Ctx* c, const KP<P>& p, int dst, int r) {
   return cudaErrorNotSupported;
 }
 
+// Whether an FP32 flight takes the ring (period_ring), by the particles a
+// warp.  Measured, rounds against ring, us a pass: 2e4 particles (5 a warp)
+// 163 against 167 (8 periods' kernels); 10 intervals of 1e6 (274) 366 against
+// 271; 1.2e6, four periods, 445 against 434; 1e7 (2741) with components 537
+// against 512, weighted 671 against 687; 1e8 (27400) 3390 against 3580.  The
+// 4D model, whose events are longer, measured slower with it at 5e7.
+constexpr long long kRingLo = 20;
+template <class F>
+constexpr long long kRingHi = F::STATIC ? 1000 : 3000;
+template <class F>
+constexpr bool kHasRing = !F::is64 && F::D == 1;
+template <class F>
+bool takes_ring(const Ctx* c) {
+  const long long n = total_n_alpha(c);
+  const long long warps = (long long)kPeriodBlocks * c->num_sms * kWarps;
+  return n >= kRingLo * warps && n < kRingHi<F> * warps;
+}
+
 // One chunk in one launch (k_period) of the model F.
-template <class F, int SRC, int DST>
+template <class F, int SRC, int DST, bool RING = false>
 cudaError_t period(Ctx* c, int l0, int L) {
+  if constexpr (kHasRing<F> && !RING) {
+    if (takes_ring<F>(c)) return period<F, SRC, DST, true>(c, l0, L);
+  }
   constexpr size_t smem = kWarps * period_warp_bytes<F>();
   struct Shape {  // once per process: more shared memory than a block may have by default
     cudaError_t err;
     int occ = 1;
     Shape() {
-      err = cudaFuncSetAttribute(k_period<F, SRC, DST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      err = cudaFuncSetAttribute(k_period<F, SRC, DST, RING>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)smem);
       if (err != cudaSuccess) return;
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_period<F, SRC, DST>, kBlock,
+      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_period<F, SRC, DST, RING>, kBlock,
                                                         smem) != cudaSuccess || occ < 1)
         occ = 1;
     }
@@ -2886,7 +3141,7 @@ cudaError_t period(Ctx* c, int l0, int L) {
   if (F::is64 && total_n_alpha(c) < 320ll * kWarps * c->num_sms && grid > c->num_sms)
     grid = c->num_sms;
   prof_begin(c);
-  k_period<F, SRC, DST><<<grid, kBlock, smem, c->stream>>>(p);
+  k_period<F, SRC, DST, RING><<<grid, kBlock, smem, c->stream>>>(p);
   prof_end(c);
   c->launches++;
   return cudaGetLastError();
