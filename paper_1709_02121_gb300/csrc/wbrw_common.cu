@@ -714,7 +714,13 @@ constexpr int kBootChunk = 1024;  // records per work item of k_boot_bin
 constexpr int kBootBinBlocks = 8; // resident blocks per SM k_boot_bin is built and launched for
 constexpr int kBootBinBatchBlocks = 6;  // the same for its batch form (shares from a table)
 constexpr int kTallyLoads = 4;          // groups of 32 records k_bootb_tally loads ahead
-constexpr int kTallyBlocks = 5;         // resident blocks per SM of k_bootb_tally (bound and grid)
+constexpr int kTallyBlocks = 3;         // resident blocks per SM of k_bootb_tally (bound and grid)
+// Shared memory of k_bootb_tally: the block's sums, then per warp a count and
+// the sums of the 16-bit halves of the weights of each (instance, side).
+constexpr size_t tally_bytes(int ninst) {
+  return (size_t)2 * ninst * (2 * 8 + (kBlock / 32) * 3 * 4);
+}
+constexpr unsigned kTallyFlush = 32768;  // records a warp sums before its 32-bit sums could overflow
 
 // The share q_i = a_i N^s / W^s of a record of side s (Alg. 2 on S^s), split
 // into its integer part and its Q0.32 residual.  fx (FP32 runs): in fixed
@@ -1014,47 +1020,56 @@ __global__ void __launch_bounds__(kBlock) k_boot_combine(const Counters* c, long
 // of salt b (a plain run is salt 0).
 // ---------------------------------------------------------------------------
 
-// Adds one run's counts and weight sums of instance i (both sides) to the
-// shared per-instance sums.
-__device__ __forceinline__ void flush_tally(unsigned long long* sn, unsigned long long* sw, int i,
-                                            unsigned long long c0, unsigned long long c1,
-                                            unsigned long long w0, unsigned long long w1) {
-  if (c0) { atomicAdd(sn + 2 * i, c0); atomicAdd(sw + 2 * i, w0); }
-  if (c1) { atomicAdd(sn + 2 * i + 1, c1); atomicAdd(sw + 2 * i + 1, w1); }
-}
-
 // N^s and W^s of every instance: its offspring records (cell | side << 31,
 // a) and its unit-weight counts (a = 2^31 each), summed per block in shared
-// memory and added to the instances' records.
+// memory and added to the instances' records.  A record adds its count and
+// the two halves of its weight to 32-bit sums of its warp in shared memory
+// (emptied into the block's 64-bit sums before they could overflow): the 32
+// records of a group belong to some eight instances (a warp's candidates come
+// from all over the batch), and summing them by shuffles over runs of equal
+// instances, with a 64-bit shared add per run, took 404 us for 3.1e7 records.
 __global__ void __launch_bounds__(kBlock, kTallyBlocks)
     k_bootb_tally(const uint32_t* rec_cell, const uint32_t* rec_a, const unsigned* rcnt, int nseg,
                   long long rseg, const int* ucnt, long long nh, int nhi, int ninst,
                   BootInst* bi) {
   const unsigned long long mag = inst_magic(nhi);
-  __shared__ unsigned long long sn[2 * kMaxInst], sw[2 * kMaxInst];
-  for (int i = threadIdx.x; i < 2 * ninst; i += kBlock) sn[i] = sw[i] = 0;
-  __syncthreads();
+  extern __shared__ unsigned long long s_tally[];
+  const int ns = 2 * ninst;
+  unsigned long long *sn = s_tally, *sw = s_tally + ns;
+  unsigned* const mine = (unsigned*)(s_tally + 2 * ns) + (threadIdx.x >> 5) * 3 * ns;
   const int lane = threadIdx.x & 31;
+  for (int i = threadIdx.x; i < ns; i += kBlock) sn[i] = sw[i] = 0;
+  for (int i = lane; i < 3 * ns; i += 32) mine[i] = 0u;
+  __syncthreads();
+  auto flush = [&]() {
+    __syncwarp();
+    for (int i = lane; i < ns; i += 32) {
+      const unsigned n = mine[i];
+      if (n) {
+        atomicAdd(sn + i, (unsigned long long)n);
+        atomicAdd(sw + i, ((unsigned long long)mine[2 * ns + i] << 16) + mine[ns + i]);
+        mine[i] = mine[ns + i] = mine[2 * ns + i] = 0u;
+      }
+    }
+    __syncwarp();
+  };
   const long long gw = ((long long)blockIdx.x * kBlock + threadIdx.x) >> 5;
   const long long nw = ((long long)gridDim.x * kBlock) >> 5;
   const long long cps = (rseg + kBootChunk - 1) / kBootChunk;
+  unsigned held = 0;
   for (long long it = gw; it < (long long)nseg * cps; it += nw) {
     const long long sg = it / cps;
     const unsigned b0 = (unsigned)((it - sg * cps) * kBootChunk);
     const unsigned n = min(min(rcnt[sg], (unsigned)rseg), b0 + (unsigned)kBootChunk);
-    // a segment holds runs of one instance's records (of both signs, the
-    // pairs interleaved)
+    if (n <= b0) continue;
+    if (held + (n - b0) > kTallyFlush) {
+      flush();
+      held = 0;
+    }
+    held += n - b0;
     const uint32_t* rcs = rec_cell + sg * rseg;
     const uint32_t* ras = rec_a + sg * rseg;
-    // kTallyLoads groups of 32 records are loaded before the first is used,
-    // so that each warp keeps that many loads in flight (the kernel streams
-    // the records once).  While consecutive groups belong to one instance
-    // their sums stay in registers (the same in every lane); they go to the
-    // block's shared sums when another instance's group comes and at the end
-    // of the chunk.
-    int cur = -1;
-    unsigned rc0 = 0, rc1 = 0;
-    unsigned long long rw0 = 0, rw1 = 0;
+    // kTallyLoads groups of 32 records are loaded before the first is used
     for (unsigned b = b0; b < n; b += 32u * kTallyLoads) {
       uint32_t rcv[kTallyLoads], rav[kTallyLoads];
 #pragma unroll
@@ -1065,63 +1080,16 @@ __global__ void __launch_bounds__(kBlock, kTallyBlocks)
       }
 #pragma unroll
       for (int j = 0; j < kTallyLoads; ++j) {
-        if (b + 32u * j >= n) break;  // warp-uniform: lane 0's record exists below
-        const bool valid = rcv[j] != ~0u;
-        const int side = (int)(rcv[j] >> 31);
-        const int inst = valid ? (int)inst_of_cell(rcv[j] & 0x7FFFFFFFu, nhi, mag) : -1;
-        const unsigned a = rav[j];
-        const int inst0 = __shfl_sync(0xFFFFFFFFu, inst, 0);
-        if (__all_sync(0xFFFFFFFFu, inst == inst0 || inst < 0)) {
-          // the warp's records belong to one instance: counts by ballots,
-          // weight sums in 16-bit halves
-          const bool s0 = valid && side == 0, s1 = valid && side == 1;
-          const unsigned c0 = __popc(__ballot_sync(0xFFFFFFFFu, s0));
-          const unsigned c1 = __popc(__ballot_sync(0xFFFFFFFFu, s1));
-          const unsigned lo0 = __reduce_add_sync(0xFFFFFFFFu, s0 ? a & 0xFFFFu : 0u);
-          const unsigned hi0 = __reduce_add_sync(0xFFFFFFFFu, s0 ? a >> 16 : 0u);
-          const unsigned lo1 = __reduce_add_sync(0xFFFFFFFFu, s1 ? a & 0xFFFFu : 0u);
-          const unsigned hi1 = __reduce_add_sync(0xFFFFFFFFu, s1 ? a >> 16 : 0u);
-          const unsigned long long w0 = ((unsigned long long)hi0 << 16) + lo0;
-          const unsigned long long w1 = ((unsigned long long)hi1 << 16) + lo1;
-          if (inst0 != cur) {  // a new run: the last one to the shared sums
-            if (lane == 0 && cur >= 0) flush_tally(sn, sw, cur, rc0, rc1, rw0, rw1);
-            cur = inst0;
-            rc0 = rc1 = 0;
-            rw0 = rw1 = 0;
-          }
-          rc0 += c0;
-          rc1 += c1;
-          rw0 += w0;
-          rw1 += w1;
-          continue;
-        }
-        // mixed instances: runs of equal instances in consecutive lanes, each
-        // run's first lane adding the run's sums
-        unsigned c0 = valid && side == 0, c1 = valid && side == 1;
-        unsigned long long w0 = c0 ? a : 0ull, w1 = c1 ? a : 0ull;
-        const int prev = __shfl_up_sync(0xFFFFFFFFu, inst, 1);
-        const bool head = lane == 0 || prev != inst;
-        const unsigned heads = __ballot_sync(0xFFFFFFFFu, head);
-        const unsigned later = heads & ~((2u << lane) - 1u);
-        const int end = later ? __ffs(later) - 1 : 32;  // the next run's first lane
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-          const unsigned d0 = __shfl_down_sync(0xFFFFFFFFu, c0, off);
-          const unsigned d1 = __shfl_down_sync(0xFFFFFFFFu, c1, off);
-          const unsigned long long v0 = __shfl_down_sync(0xFFFFFFFFu, w0, off);
-          const unsigned long long v1 = __shfl_down_sync(0xFFFFFFFFu, w1, off);
-          if (lane + off < end) {
-            c0 += d0;
-            c1 += d1;
-            w0 += v0;
-            w1 += v1;
-          }
-        }
-        if (head && inst >= 0) flush_tally(sn, sw, inst, c0, c1, w0, w1);
+        if (rcv[j] == ~0u) continue;
+        const unsigned key =
+            2u * inst_of_cell(rcv[j] & 0x7FFFFFFFu, nhi, mag) + (rcv[j] >> 31);
+        atomicAdd(mine + key, 1u);
+        atomicAdd(mine + ns + key, rav[j] & 0xFFFFu);
+        atomicAdd(mine + 2 * ns + key, rav[j] >> 16);
       }
     }
-    if (lane == 0 && cur >= 0) flush_tally(sn, sw, cur, rc0, rc1, rw0, rw1);
   }
+  flush();
   // unit counts: warps over consecutive cells
   for (long long c0 = gw * 32; c0 < nh; c0 += nw * 32) {
     const long long nu = c0 + lane;
@@ -1703,7 +1671,11 @@ static cudaError_t launch_boot_batch(Ctx* c, int epoch_delta) {
   const int fx = c->cfg.precision == WBRW_FP32;
   cudaError_t e = launch_zero(c, c->boot_inst, (size_t)ni * sizeof(BootInst));
   if (e != cudaSuccess) return e;
-  k_bootb_tally<<<grid_cap(c, kTallyBlocks), kBlock, 0, c->stream>>>(
+  static const cudaError_t tally_attr =
+      cudaFuncSetAttribute(k_bootb_tally, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)tally_bytes(kMaxInst));
+  if (tally_attr != cudaSuccess) return tally_attr;
+  k_bootb_tally<<<grid_cap(c, kTallyBlocks), kBlock, tally_bytes(ni), c->stream>>>(
       c->rec_cell, c->rec_a, c->rcnt, c->nseg, c->rseg, c->boot_ucnt, nh, nhi, ni, c->boot_inst);
   k_bootb_share<<<1, kBlock, 0, c->stream>>>(c->boot_inst, ni, fx);
   k_bootb_unit<<<grid_cap(c, 8), kBlock, 0, c->stream>>>(c->boot_inst, c->boot_ucnt, nh, nhi,
