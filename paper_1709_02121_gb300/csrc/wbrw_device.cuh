@@ -2862,6 +2862,10 @@ __global__ void __launch_bounds__(kBlock) k_init(const KP<P> p, const InitInst* 
     }
     p.s[i] = 1;
     if (p.w) p.w[i] = (T)1;
+    if constexpr (P::TG) {
+      p.tan[i] = 0.0;
+      p.tan[p.capacity + i] = 0.0;
+    }
   }
 }
 

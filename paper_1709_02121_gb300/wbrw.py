@@ -435,7 +435,7 @@ class Simulation:
         self.k = torch.empty(nd * self.capacity, dtype=fdt, device=dev)
         self.s = torch.empty(self.capacity, dtype=torch.int8, device=dev)
         self.w = torch.empty(self.capacity, dtype=fdt, device=dev) if strat != SP1_PAIR else None
-        self.tan = (torch.zeros(2 * self.capacity, dtype=torch.float64, device=dev)
+        self.tan = (torch.empty(2 * self.capacity, dtype=torch.float64, device=dev)
                     if wl.get("tangent") else None)
         self.cells = (self.nx * self.nx * self.nk * self.nk if self.dim == 4
                       else self.nx * self.nk)
