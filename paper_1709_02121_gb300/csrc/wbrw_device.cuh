@@ -327,6 +327,7 @@ struct KP {
   int strategy;     // 1 = sp1, 2 = sp2
   int l0, L;        // the intervals [l0, L) of the chunk (read at kernel entry)
   int len;          // L - l0
+  int host_period;  // l0, L and regen_base hold; else the device's period state
   unsigned long long regen_base;  // epoch << 40 of the histogram's particles
   T* x;             // coordinate d of slot i at x[d capacity + i]
   T* k;
@@ -380,13 +381,16 @@ struct KP {
 // The chunk's first interval and the regeneration's id base are
 // device-resident (Counters::per_*): the chunk set-up writes them, and a
 // captured period advances them in place, so that one captured period replays
-// correctly.  Each kernel takes them into its own copy of the parameters.
+// correctly.  Each kernel takes them into its own copy of the parameters
+// (unless the launch gave them, KP::host_period).
 template <class P>
 __device__ __forceinline__ KP<P> with_period(const KP<P>& q) {
   KP<P> p = q;
-  p.l0 = q.cnt->per_l0;
-  p.L = p.l0 + q.len;
-  p.regen_base = q.cnt->per_regen_base;
+  if (!q.host_period) {
+    p.l0 = q.cnt->per_l0;
+    p.L = p.l0 + q.len;
+    p.regen_base = q.cnt->per_regen_base;
+  }
   return p;
 }
 
@@ -2965,6 +2969,7 @@ KP<P> make_kp(const Ctx* c) {
   p.ttile_nz = c->ttile_nz;
   p.tinst_slot = c->tinst_slot;
   p.regen_base = (unsigned long long)c->epoch << 40;
+  p.host_period = c->host_period;
   p.x = (T*)c->buf.x;
   p.k = (T*)c->buf.k;
   p.s = c->buf.s;
@@ -3315,8 +3320,18 @@ struct DriverImpl {
   // or later; offspring start one interval after their birth, so L - l0
   // rounds drain every wave.
   static cudaError_t chunk(Ctx* c, int l0, int L, int src, int dst) {
-    cudaError_t e = launch_setup(c, c->capturing ? SETUP_CHUNK_DEV : SETUP_CHUNK,
-                                 (unsigned long long)l0, (unsigned long long)c->epoch << 40);
+    // a flight from the histogram into it needs no set-up launch: it reads no
+    // particle count, and outside a capture takes its first interval and id
+    // base from the parameters (sp2 and wp: their resampling kernels read the
+    // period state)
+    const bool bare = src == SRC_REGEN && dst == DST_BIN1;
+    cudaError_t e = cudaSuccess;
+    if (!bare)
+      e = launch_setup(c, c->capturing ? SETUP_CHUNK_DEV : SETUP_CHUNK,
+                       (unsigned long long)l0, (unsigned long long)c->epoch << 40);
+    else if (!c->capturing)
+      c->dev_period_ok = 0;  // the device's period state stays behind
+    c->host_period = bare && !c->capturing;
     if (e != cudaSuccess) return e;
     KP<P> p = make_kp<P>(c);
     p.l0 = l0;
@@ -3372,6 +3387,7 @@ struct DriverImpl {
                                  (unsigned long long)c->epoch << 40);
     if (e != cudaSuccess) return e;
     KP<P> p = make_kp<P>(c);
+    p.host_period = 0;
     p.grid = grid;
     p.count_ledger = count_ledger;
     if (!count_ledger) p.dgrid[0] = p.dgrid[1] = nullptr;  // observables only
@@ -3383,6 +3399,7 @@ struct DriverImpl {
                                  (unsigned long long)c->step);
     if (e != cudaSuccess) return e;
     KP<P> p = make_kp<P>(c);
+    p.host_period = 0;
     e = flight<P, SRC_REGEN, DST_ARRAY>(c, p);
     if constexpr (P::TG) {  // the tangent particles, appended
       if (e == cudaSuccess) e = flight<P, SRC_TREGEN, DST_ARRAY>(c, p);

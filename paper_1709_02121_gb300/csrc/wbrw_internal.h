@@ -267,6 +267,7 @@ struct Ctx {
   int graph_on;       // wbrw_graph: replay periods from CUDA graphs
   int one_launch;     // wbrw_one_launch_periods: fused periods where the kernels allow
   int dev_period_ok;  // the device period state equals (step, epoch)
+  int host_period;    // the chunk being launched carries its own (no set-up launch)
   int ngraphs;
   PeriodGraph graphs[kMaxGraphs];
   // placeholders of the captured event records: the first wave, then the
