@@ -276,14 +276,17 @@ __global__ void __launch_bounds__(kBlock) k_plan_a(const S src, long long nh, in
   const int t0 = blockIdx.x * per, t1 = min(t0 + per, nsub);
   unsigned long long run_s = 0;
   unsigned run_z = 0;
-  for (int t = t0; t < t1; ++t) {
+  typename S::V v[kScanItems];
+  auto fetch = [&](int t) {
     const long long base = (long long)t * kScanTile + threadIdx.x;
-    typename S::V v[kScanItems];
 #pragma unroll
     for (int i = 0; i < kScanItems; ++i) {
       const long long cell = base + i * kBlock;
       v[i] = cell < nh ? src.load(cell) : S::none();
     }
+  };
+  if (t0 < t1) fetch(t0);
+  for (int t = t0; t < t1; ++t) {
     unsigned long long s = 0;
     unsigned z = 0;
 #pragma unroll
@@ -292,6 +295,7 @@ __global__ void __launch_bounds__(kBlock) k_plan_a(const S src, long long nh, in
       s += n;
       z += n != 0;
     }
+    if (t + 1 < t1) fetch(t + 1);  // on their way while this sub-tile is summed
     z = __reduce_add_sync(0xFFFFFFFFu, z);
     s = z ? warp_sum(s) : 0ull;
     const int k = (t - t0) & 1;  // two buffers: one barrier per sub-tile
@@ -477,7 +481,10 @@ __global__ void __launch_bounds__(kBlock) k_plan_c(const S src, long long nh, in
       all_s += ss[k][i];
     }
     k ^= 1;  // two buffers: one barrier per sub-tile
-    const bool bounds = ninst > 1 || t == 0;
+    // an instance begins in this sub-tile
+    const bool bounds =
+        t == 0 || inst_of_cell((unsigned)(end - 1), nhi, mag) !=
+                      inst_of_cell((unsigned)(base - 1), nhi, mag);
     const unsigned z0 = (unsigned)g.b + st.z + pre_z;
     if (z == 0 && !bounds) continue;
     if (all_s < (1ull << 32))
