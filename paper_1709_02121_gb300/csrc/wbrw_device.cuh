@@ -1779,7 +1779,9 @@ __device__ __forceinline__ void flight_body(const KP<P>& p, WarpCounts& wc, Acc&
     // activity tests of the whole flight from the common path
     // one instance: a slot's regeneration draw depends on the slot alone, so
     // the draw of the warp's next tile is made while this tile is processed
-    constexpr bool PIPE = P::SINGLE && SRC == SRC_REGEN;
+    // (not with sp2's record tallies, whose registers it would spill: 3e7
+    // particles 3.45 against 3.27 ms a period)
+    constexpr bool PIPE = P::SINGLE && SRC == SRC_REGEN && DST != DST_BIN2;
     uint4 r_next = make_uint4(0u, 0u, 0u, 0u);
     if constexpr (PIPE) {
       const unsigned long long q0 = p.regen_base | (unsigned long long)(first + (IX)lane);
@@ -3104,11 +3106,12 @@ cudaError_t events_any(Ctx* c, const KP<P>& p, int dst, int r) {
 // warp.  Measured, rounds against ring, us a pass: 2e4 particles (5 a warp)
 // 163 against 167 (8 periods' kernels); 10 intervals of 1e6 (274) 366 against
 // 271; 1.2e6, four periods, 445 against 434; 1e7 (2741) with components 537
-// against 512, weighted 671 against 687; 1e8 (27400) 3390 against 3580.  The
+// against 512, weighted 671 against 687; 1e8 (27400) 3390 against 3580; a tangent
+// period of 4e6 (1096) 244 against 234.  The
 // 4D model, whose events are longer, measured slower with it at 5e7.
 constexpr long long kRingLo = 20;
 template <class F>
-constexpr long long kRingHi = F::STATIC ? 1000 : 3000;
+constexpr long long kRingHi = F::STATIC && !F::TG ? 1000 : 3000;
 template <class F>
 constexpr bool kHasRing = !F::is64 && F::D == 1;
 template <class F>
