@@ -956,9 +956,113 @@ __global__ void __launch_bounds__(kBlock) k_boot_guide(const Counters* c, long l
   }
 }
 
-// N_r^s = N^s - sum floor(q_i) draws per side, each an upper-bound search of
-// U = floor(r R / 2^64) in the inclusive residual prefix, within the range
-// the guide table gives.
+// N_r^s of both sides (N^s less the kept integer parts; none without a
+// residual).
+__device__ __forceinline__ void residual_draws(const Counters* c, unsigned long long* nr) {
+  for (int s = 0; s < 2; ++s) {
+    const long long d = (long long)c->boot_n[s] - (long long)c->boot_keep[s];
+    nr[s] = d > 0 ? (unsigned long long)d : 0ull;
+    if (c->boot_R[s] == 0) nr[s] = 0;
+  }
+}
+
+// The cell of a residual draw r64: an upper-bound search of U =
+// floor(r R / 2^64) in the inclusive residual prefix, within the range the
+// guide table gives for its bucket.
+__device__ __forceinline__ int draw_cell(unsigned long long r64, unsigned long long R,
+                                         const unsigned long long* pre, const int* gs) {
+  const unsigned long long U = __umul64hi(r64, R);
+  const int j = (int)(r64 >> (64 - kGuideBits));
+  int lo = gs[j], hi = gs[j + 1];  // first cell with pre > U (nh < 2^31)
+  while (lo < hi) {
+    const int mid = lo + ((hi - lo) >> 1);
+    if (pre[mid] > U) hi = mid; else lo = mid + 1;
+  }
+  return lo;
+}
+
+// The draws of large runs.  One reduction in L2 per draw bounds k_boot_draw
+// (5.5e7 draws in 0.75 ms), but most draws fall into buckets of the guide
+// table that lie in a single cell.  Those are counted by bucket in shared
+// memory (16 bits each: a block's share of the draws falls evenly into 2^16
+// buckets whatever the residuals are, at most 215 a bucket for the largest
+// capacity, 4400 standard deviations below 2^16) and added to their cells at
+// the end; the others wait until a warp has 32 of them to search.
+constexpr int kDrawBlock = 1024;  // one block per SM
+constexpr long long kDrawBuckets = 4000000;  // N_alpha from which it is taken
+constexpr size_t kDrawSmem =
+    (size_t)kGuide * 2 + kGuide / 8 + (size_t)(kDrawBlock / 32) * 64 * sizeof(unsigned long long);
+__global__ void __launch_bounds__(kDrawBlock, 1)
+    k_boot_draw_buckets(Counters* c, const unsigned long long* pre0,
+                        const unsigned long long* pre1, int* keep0, int* keep1, const int* guide,
+                        uint32_t key0, uint32_t key1, int epoch_delta) {
+  extern __shared__ unsigned long long s_draw[];
+  unsigned long long* const buf = s_draw + (threadIdx.x >> 5) * 64;
+  unsigned* const hist = (unsigned*)(s_draw + (kDrawBlock / 32) * 64);
+  unsigned* const inside = hist + kGuide / 2;
+  const int lane = threadIdx.x & 31;
+  const unsigned long long epoch = (c->per_regen_base >> 40) + (unsigned long long)epoch_delta;
+  unsigned long long nr[2];
+  residual_draws(c, nr);
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    c->boot_nr[0] = nr[0];
+    c->boot_nr[1] = nr[1];
+  }
+  for (int side = 0; side < 2; ++side) {
+    const unsigned long long n = side ? nr[1] : nr[0];
+    const unsigned long long R = c->boot_R[side];
+    const unsigned long long* const pre = side ? pre1 : pre0;
+    int* const keep = side ? keep1 : keep0;
+    const int* const gs = guide + side * (kGuide + 1);
+    __syncthreads();
+    for (int j = threadIdx.x; j < kGuide; j += kDrawBlock) {
+      const unsigned in = __ballot_sync(0xFFFFFFFFu, gs[j] == gs[j + 1]);
+      if (lane == 0) inside[j >> 5] = in;
+      if (j < kGuide / 2) hist[j] = 0u;
+    }
+    __syncthreads();
+    unsigned held = 0;  // draws to search (the same in every lane)
+    auto search = [&](unsigned take) {
+      __syncwarp();
+      if ((unsigned)lane < take)
+        atomicAdd(keep + draw_cell(buf[held - take + lane], R, pre, gs), 1);
+      __syncwarp();
+      held -= take;
+    };
+    const unsigned long long step = (unsigned long long)gridDim.x * kDrawBlock;
+    for (unsigned long long d0 = (unsigned long long)blockIdx.x * kDrawBlock +
+                                 (threadIdx.x & ~31u);
+         d0 < n; d0 += step) {
+      const unsigned long long d = d0 + lane;
+      const uint4 r = philox((uint32_t)d, (uint32_t)(d >> 32), kStepBoot,
+                             (uint32_t)((epoch << 1) | (unsigned long long)side), key0, key1);
+      const unsigned long long r64 = ((unsigned long long)r.y << 32) | r.x;
+      const unsigned j = r.y >> (32 - kGuideBits);
+      const bool in = (inside[j >> 5] >> (j & 31u)) & 1u;
+      if (d < n && in) atomicAdd(hist + (j >> 1), 1u << (16u * (j & 1u)));
+      const unsigned out = __ballot_sync(0xFFFFFFFFu, d < n && !in);
+      if (d < n && !in) buf[held + __popc(out & ((1u << lane) - 1u))] = r64;
+      held += __popc(out);
+      if (held >= 32u) search(32u);
+    }
+    if (held) search(held);
+    __syncthreads();
+    for (int i = threadIdx.x; i < kGuide / 2; i += kDrawBlock) {
+      const unsigned w = hist[i];
+      if (!w) continue;
+      const int a = (int)(w & 0xFFFFu), b = (int)(w >> 16);
+      const int ca = gs[2 * i], cb = gs[2 * i + 1];
+      if (a && b && ca == cb) {
+        atomicAdd(keep + ca, a + b);
+      } else {
+        if (a) atomicAdd(keep + ca, a);
+        if (b) atomicAdd(keep + cb, b);
+      }
+    }
+  }
+}
+
+// N_r^s draws per side, one reduction each.
 __global__ void __launch_bounds__(kBlock) k_boot_draw(Counters* c, long long nh,
                                                       const unsigned long long* pre0,
                                                       const unsigned long long* pre1,
@@ -967,11 +1071,7 @@ __global__ void __launch_bounds__(kBlock) k_boot_draw(Counters* c, long long nh,
                                                       uint32_t key1, int epoch_delta) {
   const unsigned long long epoch = (c->per_regen_base >> 40) + (unsigned long long)epoch_delta;
   unsigned long long nr[2];
-  for (int s = 0; s < 2; ++s) {
-    const long long d = (long long)c->boot_n[s] - (long long)c->boot_keep[s];
-    nr[s] = d > 0 ? (unsigned long long)d : 0ull;
-    if (c->boot_R[s] == 0) nr[s] = 0;
-  }
+  residual_draws(c, nr);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     c->boot_nr[0] = nr[0];
     c->boot_nr[1] = nr[1];
@@ -984,16 +1084,8 @@ __global__ void __launch_bounds__(kBlock) k_boot_draw(Counters* c, long long nh,
     const uint4 r = philox((uint32_t)d, (uint32_t)(d >> 32), kStepBoot,
                            (uint32_t)((epoch << 1) | (unsigned long long)side), key0, key1);
     const unsigned long long r64 = ((unsigned long long)r.y << 32) | r.x;
-    const unsigned long long U = __umul64hi(r64, c->boot_R[side]);
-    const unsigned long long* pre = side ? pre1 : pre0;
-    const int* gs = guide + side * (kGuide + 1);
-    const int j = (int)(r64 >> (64 - kGuideBits));
-    int lo = gs[j], hi = gs[j + 1];  // first cell with pre > U (nh < 2^31)
-    while (lo < hi) {
-      const int mid = lo + ((hi - lo) >> 1);
-      if (pre[mid] > U) hi = mid; else lo = mid + 1;
-    }
-    atomicAdd((side ? keep1 : keep0) + lo, 1);
+    const int cell = draw_cell(r64, c->boot_R[side], side ? pre1 : pre0, guide + side * (kGuide + 1));
+    atomicAdd((side ? keep1 : keep0) + cell, 1);
   }
 }
 
@@ -1732,9 +1824,18 @@ cudaError_t launch_boot(Ctx* c, int epoch_delta) {
   launch_residual_prefix(c);
   k_boot_guide<<<(2 * (kGuide + 1) + kBlock - 1) / kBlock, kBlock, 0, c->stream>>>(
       c->cnt, nh, c->boot_res[0], c->boot_res[1], c->boot_guide);
-  k_boot_draw<<<g, kBlock, 0, c->stream>>>(
-      c->cnt, nh, c->boot_res[0], c->boot_res[1], c->boot_keep[0], c->boot_keep[1], c->boot_guide,
-      key0, key1, epoch_delta);
+  if (c->ih[0].n_alpha >= kDrawBuckets) {
+    static const cudaError_t draw_attr = cudaFuncSetAttribute(
+        k_boot_draw_buckets, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDrawSmem);
+    if (draw_attr != cudaSuccess) return draw_attr;
+    k_boot_draw_buckets<<<c->num_sms, kDrawBlock, kDrawSmem, c->stream>>>(
+        c->cnt, c->boot_res[0], c->boot_res[1], c->boot_keep[0], c->boot_keep[1], c->boot_guide,
+        key0, key1, epoch_delta);
+  } else {
+    k_boot_draw<<<g, kBlock, 0, c->stream>>>(c->cnt, nh, c->boot_res[0], c->boot_res[1],
+                                             c->boot_keep[0], c->boot_keep[1], c->boot_guide, key0,
+                                             key1, epoch_delta);
+  }
   k_boot_combine<<<g, kBlock, 0, c->stream>>>(c->cnt, nh, c->boot_keep[0], c->boot_keep[1],
                                               c->buf.grid, key0, key1, epoch_delta);
   c->launches += 3;
