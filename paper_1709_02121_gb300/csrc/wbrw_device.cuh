@@ -2830,6 +2830,58 @@ __global__ void __launch_bounds__(kBlock, (max_blocks<P, DST>())) k_drain(const 
   reduce_event_tallies(red, acc, p.cnt, DST == DST_BIN2);
 }
 
+// The signed histogram of the arrays' particles for grids that fit shared
+// memory (one instance, 2D): a block sums its share there and adds its
+// occupied cells to the grid.  The arrays are in no order of cells, so nearly
+// every particle was a reduction of its own in L2, thousands of them on each
+// of the packet's cells (1e6 particles on 240 x 128 cells: 14 against 66 us).
+constexpr int kBinBlock = 1024;               // one block per SM
+constexpr size_t kBinSmem = 200 * 1024;       // most shared memory: 51200 cells
+constexpr long long kBinSmall = 100000;       // N_alpha from which it is taken
+template <class P>
+__global__ void __launch_bounds__(kBinBlock, 1) k_bin_small(const KP<P> p, int nh) {
+  using T = typename P::T;
+  extern __shared__ int s_hist[];
+  for (int i = threadIdx.x; i < nh; i += kBinBlock) s_hist[i] = 0;
+  __syncthreads();
+  const unsigned long long n = p.cnt->n_src;
+  Acc acc;
+  acc.zero();
+  constexpr int U = 4;  // particles a thread has in flight
+  const unsigned long long step = (unsigned long long)gridDim.x * kBinBlock;
+  for (unsigned long long i0 = (unsigned long long)blockIdx.x * kBinBlock + threadIdx.x; i0 < n;
+       i0 += U * step) {
+    PV<P> x[U], k[U];
+    T w[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const unsigned long long i = i0 + u * step;
+      const bool in = i < n;
+      x[u].c[0] = in ? p.x[i] : (T)0;
+      k[u].c[0] = in ? p.k[i] : (T)0;
+      w[u] = !in ? (T)0 : (p.w ? p.w[i] : (T)p.s[i]);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (i0 + u * step >= n) break;
+      int cell;
+      if (cell_of<P>(p, x[u], k[u], cell)) atomicAdd(s_hist + cell, is_pos(w[u]) ? 1 : -1);
+      else tally_out<P>(p, acc, w[u], x[u], k[u]);
+    }
+  }
+  const unsigned out_p = __reduce_add_sync(kFull, acc.out_p);
+  const unsigned out_m = __reduce_add_sync(kFull, acc.out_m);
+  if ((threadIdx.x & 31) == 0) {
+    if (out_p) atomicAdd(&p.cnt->ledger[LG_OUT_P], (unsigned long long)out_p);
+    if (out_m) atomicAdd(&p.cnt->ledger[LG_OUT_M], (unsigned long long)out_m);
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < nh; i += kBinBlock) {
+    const int v = s_hist[i];
+    if (v) atomicAdd(p.grid + i, v);
+  }
+}
+
 // Initial particles from the Gaussian-wavepacket Wigner function (positive):
 // Box-Muller on the init stream of pid = (instance << 32) | index, with
 // x ~ N(x0, sx^2), k ~ N(k0, sk^2) of the slot's instance.
@@ -3394,6 +3446,17 @@ struct DriverImpl {
     p.grid = grid;
     p.count_ledger = count_ledger;
     if (!count_ledger) p.dgrid[0] = p.dgrid[1] = nullptr;  // observables only
+    if constexpr (P::D == 1 && !P::TG) {
+      const size_t smem = (size_t)c->nh * sizeof(int);
+      if (dst == DST_BIN1 && c->ninst == 1 && smem <= kBinSmem && c->ih[0].n_alpha >= kBinSmall) {
+        static const cudaError_t attr = cudaFuncSetAttribute(
+            k_bin_small<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBinSmem);
+        if (attr != cudaSuccess) return attr;
+        k_bin_small<P><<<c->num_sms, kBinBlock, smem, c->stream>>>(p, (int)c->nh);
+        c->launches++;
+        return cudaGetLastError();
+      }
+    }
     return flight_any<P>(c, p, SRC_ARRAY, dst);
   }
 
