@@ -289,6 +289,21 @@ wbrw_status resample_from_arrays(wbrw_ctx* c) {
   return WBRW_OK;
 }
 
+// The advance of a captured period's device state by len intervals, on the
+// side branch: nothing after an sp1 flight reads that state, so the plan need
+// not wait for it (the branch is joined before the capture ends).
+cudaError_t advance_beside(wbrw_ctx* c, int len) {
+  cudaError_t e = cudaEventRecord(c->prof_fork, c->stream);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(c->prof_side, c->prof_fork, 0);
+  if (e != cudaSuccess) return e;
+  const cudaStream_t main = c->stream;
+  c->stream = c->prof_side;
+  e = launch_setup(c, SETUP_ADVANCE, (unsigned long long)len, 0);
+  c->stream = main;
+  c->prof_side_used = 1;
+  return e;
+}
+
 // One fused period of wbrw_run: zero the histogram (sp1) or the bootstrap
 // tallies (sp2), fly [l0, L) from src into the sink, bootstrap (sp2), and
 // build the regeneration plan.  The source's ids are those of regen_epoch;
@@ -315,6 +330,8 @@ wbrw_status enqueue_period(wbrw_ctx* c, int src, int l0, int L, long long regen_
   cudaError_t e = d->chunk(c, l0, L, src, dst);
   c->epoch = keep_epoch;
   WBRW_TRY(c, e, "period");
+  if (c->capturing && c->cfg.strategy == WBRW_SP1_PAIR)
+    WBRW_TRY(c, advance_beside(c, L - l0), "advance");
   // the device id base is still the source's epoch: the histogram is the next
   if (c->cfg.strategy == WBRW_SP2_BOOTSTRAP) WBRW_TRY(c, launch_boot(c, 1), "bootstrap");
   if (c->cfg.strategy == WBRW_WP) WBRW_TRY(c, launch_wp_round(c, 1), "rounding");
@@ -344,7 +361,7 @@ wbrw_status capture_period(wbrw_ctx* c, int len, PeriodGraph* g) {
            "begin capture");
   c->capturing = 1;
   wbrw_status st = enqueue_period(c, SRC_REGEN, (int)c->step, (int)c->step + len, c->epoch);
-  if (st == WBRW_OK)
+  if (st == WBRW_OK && c->cfg.strategy != WBRW_SP1_PAIR)
     st = cuda_check(c, launch_setup(c, SETUP_ADVANCE, (unsigned long long)len, 0), "advance");
   if (c->prof_side_used) {  // join the profiling branch before the capture ends
     cudaEventRecord(c->prof_join, c->prof_side);
