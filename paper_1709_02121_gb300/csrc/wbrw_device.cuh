@@ -314,6 +314,7 @@ struct KP {
   long long kmin_ord, kmax_ord;  // FP64: ordered(), a zero bound as -0
   int nx, nk;
   float inv_nk;     // 1/nk, for cell -> (ix, ik)
+  uint32_t nk_mag, nx_mag;  // ceil(2^32 / nk), ceil(2^32 / nx) (4D; 0 for 1)
   int nh_big;       // cells per instance >= 2^24: an integer division instead
   unsigned long long inst_mag;  // ceil(2^40 / nhi): the instance of a global cell
   int ninst;        // instances in the batch (1 for a single run)
@@ -1335,6 +1336,19 @@ __device__ __forceinline__ typename P::T in_cell(typename P::T v, typename P::T 
   return v;
 }
 
+// v = q d + r for 0 <= v < 2^30 from m = ceil(2^32 / d) (d > 1): the product's
+// high word is the quotient or one more (v (m - 2^32 / d) < 2^30).  An
+// integer division by a divisor known only at run time costs some four times
+// the instructions, and a regenerated 4D particle takes three.
+__device__ __forceinline__ void divide(int v, int d, uint32_t m, int& q, int& r) {
+  q = d > 1 ? (int)__umulhi((unsigned)v, m) : v;
+  r = v - q * d;
+  if (r < 0) {
+    --q;
+    r += d;
+  }
+}
+
 // Instance of a slot of the base region: the last instance whose first slot
 // is <= slot (empty instances share their start with the next one).
 template <class P>
@@ -1861,9 +1875,10 @@ __device__ __forceinline__ void flight_body(const KP<P>& p, WarpCounts& wc, Acc&
             // cell = ((ix1 nx + ix2) nk + ik1) nk + ik2; x offsets from the
             // draw (pid, REGEN, 0), k offsets from (pid, REGEN, 1) in FP64,
             // all four from the first draw in FP32
-            const int ik2 = cell % p.nk, c1 = cell / p.nk;
-            const int ik1 = c1 % p.nk, c2 = c1 / p.nk;
-            const int ix2 = c2 % p.nx, ix1 = c2 / p.nx;
+            int c1, ik2, c2, ik1, ix1, ix2;
+            divide(cell, p.nk, p.nk_mag, c1, ik2);
+            divide(c1, p.nk, p.nk_mag, c2, ik1);
+            divide(c2, p.nx, p.nx_mag, ix1, ix2);
             T u[4];
             if constexpr (P::is64) {
               const uint4 r2 = philox_ks(p.ks, (uint32_t)pid, (uint32_t)(pid >> 32), kStepRegen, 1u);
@@ -2984,6 +2999,8 @@ KP<P> make_kp(const Ctx* c) {
   p.nx = g.nx;
   p.nk = g.nk;
   p.inv_nk = 1.0f / (float)g.nk;
+  p.nk_mag = g.nk > 1 ? (uint32_t)(((1ull << 32) + g.nk - 1) / g.nk) : 0u;
+  p.nx_mag = g.nx > 1 ? (uint32_t)(((1ull << 32) + g.nx - 1) / g.nx) : 0u;
   p.nh_big = (long long)c->nhi >= (1ll << 24);
   p.inst_mag = ((1ull << 40) + (unsigned long long)c->nhi - 1ull) / (unsigned long long)c->nhi;
   p.ninst = c->ninst;
