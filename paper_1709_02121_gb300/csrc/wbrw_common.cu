@@ -1770,10 +1770,10 @@ static cudaError_t launch_boot_batch(Ctx* c, int epoch_delta) {
   const int fx = c->cfg.precision == WBRW_FP32;
   cudaError_t e = launch_zero(c, c->boot_inst, (size_t)ni * sizeof(BootInst));
   if (e != cudaSuccess) return e;
-  static const cudaError_t tally_attr =
-      cudaFuncSetAttribute(k_bootb_tally, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)tally_bytes(kMaxInst));
-  if (tally_attr != cudaSuccess) return tally_attr;
+  static SharedMemoryLimit limit;
+  if ((e = limit.allow((const void*)k_bootb_tally, tally_bytes(kMaxInst), c->device)) !=
+      cudaSuccess)
+    return e;
   k_bootb_tally<<<grid_cap(c, kTallyBlocks), kBlock, tally_bytes(ni), c->stream>>>(
       c->rec_cell, c->rec_a, c->rcnt, c->nseg, c->rseg, c->boot_ucnt, nh, nhi, ni, c->boot_inst);
   k_bootb_share<<<1, kBlock, 0, c->stream>>>(c->boot_inst, ni, fx);
@@ -1825,9 +1825,9 @@ cudaError_t launch_boot(Ctx* c, int epoch_delta) {
   k_boot_guide<<<(2 * (kGuide + 1) + kBlock - 1) / kBlock, kBlock, 0, c->stream>>>(
       c->cnt, nh, c->boot_res[0], c->boot_res[1], c->boot_guide);
   if (c->ih[0].n_alpha >= kDrawBuckets) {
-    static const cudaError_t draw_attr = cudaFuncSetAttribute(
-        k_boot_draw_buckets, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDrawSmem);
-    if (draw_attr != cudaSuccess) return draw_attr;
+    static SharedMemoryLimit limit;
+    const cudaError_t e = limit.allow((const void*)k_boot_draw_buckets, kDrawSmem, c->device);
+    if (e != cudaSuccess) return e;
     k_boot_draw_buckets<<<c->num_sms, kDrawBlock, kDrawSmem, c->stream>>>(
         c->cnt, c->boot_res[0], c->boot_res[1], c->boot_keep[0], c->boot_keep[1], c->boot_guide,
         key0, key1, epoch_delta);

@@ -3197,25 +3197,24 @@ cudaError_t period(Ctx* c, int l0, int L) {
     if (takes_ring<F>(c)) return period<F, SRC, DST, true>(c, l0, L);
   }
   constexpr size_t smem = kWarps * period_warp_bytes<F>();
-  struct Shape {  // once per process: more shared memory than a block may have by default
-    cudaError_t err;
-    int occ = 1;
-    Shape() {
-      err = cudaFuncSetAttribute(k_period<F, SRC, DST, RING>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem);
-      if (err != cudaSuccess) return;
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_period<F, SRC, DST, RING>, kBlock,
-                                                        smem) != cudaSuccess || occ < 1)
-        occ = 1;
-    }
-  };
-  static const Shape shape;
-  if (shape.err != cudaSuccess) return shape.err;
+  static SharedMemoryLimit limit;
+  if (smem > 0) {
+    const cudaError_t e = limit.allow((const void*)k_period<F, SRC, DST, RING>, smem, c->device);
+    if (e != cudaSuccess) return e;
+  }
+  static const int occ = [] {
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_period<F, SRC, DST, RING>,
+                                                      kBlock, smem) != cudaSuccess ||
+        per_sm < 1)
+      per_sm = 1;
+    return per_sm;
+  }();
   KP<F> p = make_kp<F>(c);
   p.l0 = l0;
   p.L = L;
   p.len = L - l0;
-  int grid = grid_of(c, shape.occ);
+  int grid = grid_of(c, occ);
   // FP64, few particles: one block per SM, whose warps then have fuller
   // passes (N_alpha = 2e5, 3 periods: 1.98 against 2.20 ms; 6e5: 4.80 against
   // 4.65 ms)
@@ -3466,9 +3465,9 @@ struct DriverImpl {
     if constexpr (P::D == 1 && !P::TG) {
       const size_t smem = (size_t)c->nh * sizeof(int);
       if (dst == DST_BIN1 && c->ninst == 1 && smem <= kBinSmem && c->ih[0].n_alpha >= kBinSmall) {
-        static const cudaError_t attr = cudaFuncSetAttribute(
-            k_bin_small<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBinSmem);
-        if (attr != cudaSuccess) return attr;
+        static SharedMemoryLimit limit;
+        if ((e = limit.allow((const void*)k_bin_small<P>, kBinSmem, c->device)) != cudaSuccess)
+          return e;
         k_bin_small<P><<<c->num_sms, kBinBlock, smem, c->stream>>>(p, (int)c->nh);
         c->launches++;
         return cudaGetLastError();

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "wbrw.h"
 
 namespace wbrw {
@@ -294,6 +296,21 @@ struct Ctx {
 };
 
 enum { ST_PARTICLES = 0, ST_HISTOGRAM = 1 };
+
+// Lets a kernel take more dynamic shared memory than a block may by default:
+// an attribute of the kernel on a device, set before its first launch there
+// (one object per kernel; any number of threads).
+struct SharedMemoryLimit {
+  std::atomic<unsigned long long> devices{0};
+  cudaError_t allow(const void* kernel, size_t bytes, int device) {
+    const unsigned long long bit = 1ull << (device & 63);
+    if (device < 64 && (devices.load(std::memory_order_acquire) & bit)) return cudaSuccess;
+    const cudaError_t e =
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess) devices.fetch_or(bit, std::memory_order_release);
+    return e;
+  }
+};
 
 
 // Per-precision drivers (wbrw_fp64.cu / wbrw_fp32.cu).
