@@ -1627,9 +1627,10 @@ __global__ void __launch_bounds__(kBlock) k_obs_over_na(unsigned long long* acc,
 __global__ void __launch_bounds__(kBlock) k_live_inst(const Counters* c,
                                                       const unsigned long long* inst_slot,
                                                       const unsigned* cinst, int inst,
+                                                      unsigned long long capacity,
                                                       unsigned long long* out) {
   __shared__ unsigned long long red[kBlock / 32 + 1];
-  const unsigned long long n = c->n, nb = c->n_base;
+  const unsigned long long n = min(c->n, capacity), nb = c->n_base;
   unsigned long long s = 0;
   for (unsigned long long i = nb + (unsigned long long)blockIdx.x * kBlock + threadIdx.x; i < n;
        i += (unsigned long long)gridDim.x * kBlock)
@@ -1917,7 +1918,8 @@ cudaError_t launch_transmission_gradients(Ctx* c) {
 }
 
 cudaError_t launch_live_instance(Ctx* c, int inst, unsigned long long* out) {
-  k_live_inst<<<grid_cap(c, 4), kBlock, 0, c->stream>>>(c->cnt, c->inst_slot, c->cinst, inst, out);
+  k_live_inst<<<grid_cap(c, 4), kBlock, 0, c->stream>>>(c->cnt, c->inst_slot, c->cinst, inst,
+                                                        (unsigned long long)c->buf.capacity, out);
   c->launches++;
   return cudaGetLastError();
 }

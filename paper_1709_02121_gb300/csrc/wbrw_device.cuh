@@ -1715,7 +1715,8 @@ struct SourceInfo {
   template <class P>
   __device__ __forceinline__ void load(const KP<P>& p) {
     if constexpr (SRC == SRC_ARRAY) {
-      n = p.cnt->n_src;
+      // (after an overflow, which is reported, the count runs past the arrays)
+      n = min(p.cnt->n_src, (unsigned long long)p.capacity);
       n_base = p.cnt->n_base;
       base_pid = p.cnt->base_pid;
     } else if constexpr (SRC == SRC_REGEN || SRC == SRC_TREGEN) {
@@ -2451,7 +2452,14 @@ __device__ __forceinline__ void period_ring(const KP<P>& p, WarpCounts& wc, Acc&
   unsigned nb = 0;            // accepted events waiting (the same in every lane)
   unsigned pf = 0, flip = 0;  // candidates from cq.head on staged in half `flip` of stage
   for (;;) {
-    const unsigned ne = min(wc.e - cq.head, 2u * cq.half), nd = min(wc.d, dcap);
+    unsigned ne = wc.e - cq.head;
+    if (ne > 2u * cq.half) {  // what found the ring full was dropped (and reported)
+      ne = 2u * cq.half;
+      __syncwarp();
+      if (lane == 0) wc.e = cq.head + ne;
+      __syncwarp();
+    }
+    const unsigned nd = min(wc.d, dcap);
     if (nb >= 32u || (nb && !nd && !ne)) {
       // the pairs of accepted events, one per lane
       const unsigned take = min(nb, 32u);
@@ -2859,7 +2867,7 @@ __global__ void __launch_bounds__(kBinBlock, 1) k_bin_small(const KP<P> p, int n
   extern __shared__ int s_hist[];
   for (int i = threadIdx.x; i < nh; i += kBinBlock) s_hist[i] = 0;
   __syncthreads();
-  const unsigned long long n = p.cnt->n_src;
+  const unsigned long long n = min(p.cnt->n_src, (unsigned long long)p.capacity);
   Acc acc;
   acc.zero();
   constexpr int U = 4;  // particles a thread has in flight
@@ -2947,7 +2955,8 @@ __global__ void __launch_bounds__(kBlock) k_init(const KP<P> p, const InitInst* 
 template <class P>
 __global__ void __launch_bounds__(kBlock) k_pids(const KP<P> p, unsigned long long* out,
                                                  unsigned* inst_out) {
-  const unsigned long long n = p.cnt->n, nb = p.cnt->n_base, bp = p.cnt->base_pid;
+  const unsigned long long n = min(p.cnt->n, (unsigned long long)p.capacity);
+  const unsigned long long nb = p.cnt->n_base, bp = p.cnt->base_pid;
   for (unsigned long long i = (unsigned long long)blockIdx.x * kBlock + threadIdx.x; i < n;
        i += (unsigned long long)gridDim.x * kBlock) {
     int inst = 0;

@@ -97,3 +97,20 @@ def test_high_rates_run_launch_per_round(torch):
         s.annihilate()
     assert np.array_equal(a.grid_counts(), b.grid_counts())
     assert a.counters()["launches"] == b.counters()["launches"]
+
+
+@pytest.mark.parametrize("n", [2000, 120_000])
+def test_a_full_queue_is_reported(torch, n):
+    """Growth beyond the capacity ends the flight with the capacity error in
+    either schedule (the excess is dropped, the launch ends by itself)."""
+    from paper_1709_02121_gb300 import Simulation, WbrwError, wbrw
+    wl = workloads.scaled(workloads.GAUSS_2D_FP64_2E5, precision="fp32", n_alpha=n, **BASE)
+    wl["resample_every"] = 0
+    for one in (True, False):
+        sim = Simulation(wl, n + 50)
+        sim.one_launch_periods(one)
+        with pytest.raises(WbrwError) as ei:
+            sim.step(9)
+            sim.density()
+        assert ei.value.status == wbrw.ERR_CAPACITY
+        sim.close()
